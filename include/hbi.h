@@ -444,7 +444,7 @@ typedef struct {
     int64_t bytes_factors;        /* packed factor + dense bytes read per HMVM (with padding) */
     int64_t bytes_algorithmic;    /* per HMVM: stored entries x element size + scales +
                                      x, y and intermediate vectors, no padding */
-    int64_t n_tasks_vt, n_tasks_uy; /* work items of the two HMVM phases */
+    int64_t n_tasks_vt, n_tasks_uy; /* work items of the two HMVM phases (UY: pieces of leaf row units) */
     int storage;
     double build_seconds;
     int64_t bytes_alg_vt;         /* algorithmic bytes of the V^T x phase: V entries, V scales,
@@ -523,7 +523,8 @@ hbi_status hbi_time_hmvm(hbi_handle *h, int n_rep, double *out4, hbi_stream stre
 /*
  * hbi_autotune -- pick this handle's HMVM launch configuration by timing it on the GPU: the
  * per-pass cost used by the V^T kernel to choose rows per pass and lanes per row for each
- * item (4, 8 or 16), and for the U t + dense kernel the rows per lane group (4 or 8) and CTAs
+ * item (4, 8 or 16), and for the U t + dense kernel the rows per lane group (4 or 8; small
+ * operators keep the 1 or 2 of their build) and CTAs
  * per SM (up to three values below the occupancy limit).  Each phase is timed as the average
  * of n_rep back-to-back launches on `stream` with the handle's current input; the fastest
  * setting is kept (until hbi_destroy) and used by every later product and by hbi_step.  The

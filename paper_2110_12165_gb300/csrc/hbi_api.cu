@@ -935,8 +935,9 @@ hbi_status hbi_autotune(hbi_handle *h, int n_rep, int *out3, double *out_ms, hbi
         best_vt = 0.0;
     }
     // UY phase: rows per pass and CTAs per SM
-    for (int v = 0; v < 2 && !st; ++v) {
-        h->uy_rpw = v ? 8 : 4;
+    const int base_rpw = h->uy_rpw_base;
+    for (int v = 0; v < (base_rpw == 4 ? 2 : 1) && !st; ++v) {
+        h->uy_rpw = v ? 8 : base_rpw;
         const int occ = h->uy_occ[v];
         for (int per_sm = occ; per_sm >= std::max(1, occ - 2) && !st; --per_sm) {
             set_uy_grid(h, per_sm);

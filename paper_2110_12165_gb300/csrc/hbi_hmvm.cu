@@ -7,7 +7,7 @@
 //               V columns), cut into row blocks and, for wide groups, column chunks whose
 //               sums stay in registers of one CTA.  Input = the contiguous x_sigma slice,
 //               staged with the panel through shared memory by TMA bulk copies.
-//   UY tasks  : one per leaf row cluster: the concatenation over every block covering those
+//   UY tasks  : pieces of the leaf row clusters, each row the concatenation over every block covering those
 //               rows of its U slice (low-rank) or its dense rows.  Input = the matching
 //               t_b and x_sigma values, gathered into shared memory.  Each output row is
 //               written exactly once, so the result needs no atomics and is bitwise
@@ -20,7 +20,7 @@
 // column of the near-field segment).  FP16/BF16 values carry one power-of-two scale per
 // factor column: U and V column scales fold into the VT output, dense column scales into the
 // UY gather, so the inner loops are plain dot products with FP32 (FP64) accumulation.
-// UY tasks are claimed from an atomic counter in decreasing size order (LPT), which keeps
+// UY tasks (pieces of leaf row units) are claimed from an atomic counter in decreasing size order (LPT), which keeps
 // the persistent grid (a multiple of the SM count) busy until the end; VT items follow a
 // static LPT schedule made on the host.
 #include <cuda_bf16.h>
@@ -43,9 +43,14 @@ namespace hbi {
 
 constexpr int GEMV_THREADS = 256;           // UY phase
 constexpr int GEMV_RPW = 4;                 // rows per lane group and pass (VT chunks)
-// UY rows per lane group and pass: 4 (registers sized for 5 CTAs per SM) or 8 (4 CTAs),
-// chosen per handle (default 4; hbi_autotune times both)
-template <int R> struct UyShape { static constexpr int blocks = R >= 8 ? 4 : 5; };
+// UY rows per lane group and pass: 4 (registers sized for 5 CTAs per SM) or 8 (4 CTAs; for
+// hbi_autotune to time against 4), and for operators cut into pieces of at most 16 / 8 rows 2 / 1,
+// so that all eight warps have rows: at 2,048 elements with pieces of 8 rows the UY phase takes
+// 12.8 us with 1 row per pass, 14.8 us with 2 or 4
+template <int R> struct UyShape {
+    static constexpr int blocks = R >= 8 ? 4 : 5;
+    static constexpr int min_lanes = R >= 8 ? 8 : 4;   // lanes of the shortest row
+};
 constexpr int VT_PASS_COST = 8;              // default per-pass cost of the VT shape choice
 constexpr int64_t VT_PANEL_BYTES = 40 << 10; // VT item panel: one shared-memory stage
 constexpr int64_t VT_X_BYTES = 8 << 10;      // VT item x slice
@@ -183,51 +188,69 @@ __device__ __forceinline__ A reduce_scatter(A (&v)[R], int sl, int lpr, int &row
 }
 
 // acc[q] += row q of a row-major segment (stride cpad) . z for q < nr <= R; the row is
-// split over `lpr` lanes (sub-lane sl), each taking 16-byte vectors lpr apart.
+// split over `lpr` lanes (sub-lane sl), each taking 16-byte vectors lpr apart.  UN column steps
+// are loaded ahead of their FMAs, so that a lane keeps eight 16-byte loads in flight whatever R
+// is; each row's FMAs stay in column order.  FULL: nr == R; else the missing rows' loads are
+// predicated off, so that the last row block of a unit streams like the others and its partial
+// sums stay in registers (UY phase at N = 160,000: 475 us against 513 us with a loop over the
+// rows present, 96 % of the copy bandwidth).
+template <int R, int UN, bool FULL, typename T>
+__device__ __forceinline__ void segment_steps(const T *__restrict__ rowp, int cpad, int nr,
+                                              const typename Vec<T>::A *z, int c, int step,
+                                              typename Vec<T>::A (&acc)[R]) {
+    using A = typename Vec<T>::A;
+    constexpr int VEC = Vec<T>::N;
+    uint4 raw[UN][R];
+#pragma unroll
+    for (int u = 0; u < UN; ++u)
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            if (FULL || q < nr) raw[u][q] = ld_stream(rowp + (size_t)q * cpad + c + u * step);
+            else raw[u][q] = make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+    for (int u = 0; u < UN; ++u) {
+        A zv[VEC];
+        load_z(z + c + u * step, zv);
+#pragma unroll
+        for (int q = 0; q < R; ++q) Vec<T>::fma(raw[u][q], zv, acc[q]);
+    }
+}
 template <int R, typename T>
 __device__ __forceinline__ void segment_dot(const T *__restrict__ rowp, int cpad, int nr, const typename Vec<T>::A *z,
                                             int sl, int lpr, typename Vec<T>::A (&acc)[R]) {
-    using A = typename Vec<T>::A;
-    constexpr int VEC = Vec<T>::N;
+    constexpr int VEC = Vec<T>::N, UN = R >= 8 ? 1 : 8 / R;
     const int step = lpr * VEC;
+    int c = sl * VEC;
     if (nr == R) {
-#pragma unroll(R >= 8 ? 1 : 2)
-        for (int c = sl * VEC; c < cpad; c += step) {
-            uint4 raw[R];
-#pragma unroll
-            for (int q = 0; q < R; ++q) raw[q] = ld_stream(rowp + (size_t)q * cpad + c);
-            A zv[VEC];
-            load_z(z + c, zv);
-#pragma unroll
-            for (int q = 0; q < R; ++q) Vec<T>::fma(raw[q], zv, acc[q]);
-        }
+        if (UN > 1)
+#pragma unroll 1
+            for (; c + (UN - 1) * step < cpad; c += UN * step)
+                segment_steps<R, UN, true, T>(rowp, cpad, nr, z, c, step, acc);
+#pragma unroll 1
+        for (; c < cpad; c += step) segment_steps<R, 1, true, T>(rowp, cpad, nr, z, c, step, acc);
     } else if (nr > 0) {
-        for (int c = sl * VEC; c < cpad; c += step) {
-            A zv[VEC];
-            load_z(z + c, zv);
-            for (int q = 0; q < nr; ++q) {
-                uint4 raw = ld_stream(rowp + (size_t)q * cpad + c);
-                Vec<T>::fma(raw, zv, acc[q]);
-            }
-        }
+#pragma unroll 1
+        for (; c < cpad; c += step) segment_steps<R, 1, false, T>(rowp, cpad, nr, z, c, step, acc);
     }
 }
 
-// One leaf row unit per task, claimed from a work counter in decreasing size order.  The
-// CTA gathers the unit's input ([x_sigma of its dense blocks | t_b of its low-rank blocks],
-// dense columns pre-multiplied by their scales) into shared memory, then every row is one
-// dot product over [dense segment | low-rank segment], written once to y.
+// One piece of a leaf row unit per task (whole elements, at most the unit), claimed from a work
+// counter in decreasing size order.  The CTA gathers the unit's input ([x_sigma of its dense
+// blocks | t_b of its low-rank blocks], dense columns pre-multiplied by their scales) into
+// shared memory, then every row is one dot product over [dense segment | low-rank segment],
+// written once to y.
 // TD = dense-segment element type, TL = low-rank-segment element type (same accumulator).
-// FUSE: once a unit's rows are written (and visible to the CTA after its barrier), the CTA
-// runs Cash-Karp stage `stage` for the unit's elements, whose product rows these are
-// (stage_elem or stage_vec_elem for stages 0-4, final_unit with the error maxima for stage 5): once the next
-// unit's input is gathered, its first FUSE_WARPS warps run the stage while the other warps
-// stream the next unit's rows, whose row blocks the warps claim from a shared-memory counter
-// so that the stage warps join them when done; the CTA runs the stage of its last unit with
-// every thread after its last claim.  The stage's FP64
-// arithmetic so overlaps the streaming instead of taking a launch of its own.  The next
-// product's input goes to ode.xt, a buffer other than xt; y is read back through ode.yp (so
-// y is not declared __restrict__).
+// FUSE: once a piece's rows are written (and visible to the CTA after its barrier), the CTA
+// runs Cash-Karp stage `stage` for the piece's elements, whose product rows these are
+// (stage_elem or stage_vec_elem for stages 0-4, final_unit with the error maxima for stage 5):
+// once the next piece's input is gathered, its first FUSE_WARPS warps run the stage while the
+// other warps stream the next piece's rows, whose row blocks the warps claim from a
+// shared-memory counter so that the stage warps join them when done; the CTA runs the stage of
+// its last piece with every thread after its last claim.  The stage's FP64 arithmetic so
+// overlaps the streaming instead of taking a launch of its own.  The next product's input goes
+// to ode.xt, a buffer other than xt; y is read back through ode.yp (so y is not declared
+// __restrict__).
 // FUSE selects the law: 0 none, 1 fixed rake (stage_elem, final_elem), 2 rake-free
 // (stage_vec_elem, final_vec_elem).
 constexpr int FUSE_WARPS = 2;
@@ -253,8 +276,9 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
     static_assert(std::is_same<typename Vec<TD>::A, A>::value, "segments must share the accumulator");
     constexpr int GU = 4;   // gather: independent index -> value chains per thread
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    A *z = reinterpret_cast<A *>(smem_raw);
-    __shared__ int s_task;
+    A *const z = reinterpret_cast<A *>(smem_raw);
+    __shared__ int s_next;          // the claimed piece
+    __shared__ int s_rowctr;        // FUSE: the piece's next row block (claimed by warps)
     if (stop != nullptr && *(volatile const int *)stop) {
         // a skipped product (every active model rejected: k_0 kept) still forms the stage
         // inputs of the new step size; once every model stopped there is nothing to do
@@ -265,16 +289,15 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
             }
         return;
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    int prev_e0 = 0, prev_ne = 0;   // FUSE: the unit whose rows this CTA wrote last
-    __shared__ int s_rowctr;        // FUSE: the unit's next row block (claimed by warps)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = GEMV_THREADS / 32;
+    int prev_e0 = 0, prev_ne = 0;   // FUSE: the piece whose rows this CTA wrote last
     for (;;) {
         if (threadIdx.x == 0) {
-            s_task = atomicAdd(counter, 1);
+            s_next = atomicAdd(counter, 1);
             if (FUSE) s_rowctr = 0;
         }
         __syncthreads();
-        const int ti = s_task;
+        const int ti = s_next;
         if (ti >= ntasks) {
             if (FUSE && prev_ne > 0) fused_stage<FUSE>(ode, stage, prev_e0, prev_ne, blockDim.x);
             // every CTA has made its last claim once all have counted themselves out here:
@@ -289,6 +312,7 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
             break;
         }
         const GemvTask tk = tasks[ti];
+        bool rows_on = mskip == nullptr || !mskip[tk.model];   // rows of a finished model: nothing to do
 #ifdef HBI_BOUNDS_CHECK
         const bool task_bad =
             threadIdx.x == 0 &&
@@ -298,63 +322,55 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
                    tk.out_off + tk.rows <= g_lim.n_y && tk.gather_off >= 0 &&
                    tk.gather_off + tk.cpad + tk.cpad_d <= g_lim.n_gather &&
                    (int64_t)(tk.cpad + tk.cpad_d) * (int64_t)sizeof(A) <= g_lim.smem_uy);
-        if (__syncthreads_or(task_bad)) {
-            if (FUSE && prev_ne > 0) fused_stage<FUSE>(ode, stage, prev_e0, prev_ne, blockDim.x);
-            prev_ne = 0;
-            __syncthreads();
-            continue;
-        }
+        rows_on = rows_on && !__syncthreads_or(task_bad);
 #endif
-        const bool rows_on = mskip == nullptr || !mskip[tk.model];   // rows of a finished model: nothing to do
         if (rows_on) {
             const int ctot = tk.cpad_d + tk.cpad;
             // ---- input gather into shared memory: [dense segment | low-rank segment]
-            {
-                const int *gi = gidx + tk.gather_off;
-                const float *gs = gscale != nullptr ? gscale + tk.gather_off : nullptr;
-                const int gn = blockDim.x;   // gathering threads
-                for (int c0 = threadIdx.x; c0 < ctot; c0 += GU * gn) {
-                    int idx[GU];
+            const int *gi = gidx + tk.gather_off;
+            const float *gs = gscale != nullptr ? gscale + tk.gather_off : nullptr;
+            for (int c0 = threadIdx.x; c0 < ctot; c0 += GU * GEMV_THREADS) {
+                int idx[GU];
 #pragma unroll
-                    for (int u = 0; u < GU; ++u) {
-                        const int c = c0 + u * gn;
-                        idx[u] = c < ctot ? gi[c] : -1;
+                for (int u = 0; u < GU; ++u) {
+                    const int c = c0 + u * GEMV_THREADS;
+                    idx[u] = c < ctot ? gi[c] : -1;
 #ifdef HBI_BOUNDS_CHECK
-                        if (HBI_BC(idx[u] == -1 || (idx[u] >= 0 && idx[u] < g_lim.n_xt) ||
-                                   (idx[u] <= -2 && -1 - (int64_t)idx[u] < g_lim.n_xt)))
-                            idx[u] = -1;
+                    if (HBI_BC(idx[u] == -1 || (idx[u] >= 0 && idx[u] < g_lim.n_xt) ||
+                               (idx[u] <= -2 && -1 - (int64_t)idx[u] < g_lim.n_xt)))
+                        idx[u] = -1;
 #endif
-                    }
-                    A v[GU];
+                }
+                A v[GU];
 #pragma unroll
-                    for (int u = 0; u < GU; ++u)   // -1: padding; <= -2: the pair at -2 - idx
-                        v[u] = idx[u] >= 0 ? xt[idx[u]] : (idx[u] <= -2 ? xt[-2 - idx[u]] + xt[-1 - idx[u]] : A(0));
-                    if (gs != nullptr) {
-#pragma unroll
-                        for (int u = 0; u < GU; ++u) {
-                            const int c = c0 + u * gn;
-                            if (c < ctot) v[u] *= (A)gs[c];
-                        }
-                    }
+                for (int u = 0; u < GU; ++u)   // -1: padding; <= -2: the pair at -2 - idx
+                    v[u] = idx[u] >= 0 ? xt[idx[u]] : (idx[u] <= -2 ? xt[-2 - idx[u]] + xt[-1 - idx[u]] : A(0));
+                if (gs != nullptr) {
 #pragma unroll
                     for (int u = 0; u < GU; ++u) {
-                        const int c = c0 + u * gn;
-                        if (c < ctot) z[c] = v[u];
+                        const int c = c0 + u * GEMV_THREADS;
+                        if (c < ctot) v[u] *= (A)gs[c];
                     }
+                }
+#pragma unroll
+                for (int u = 0; u < GU; ++u) {
+                    const int c = c0 + u * GEMV_THREADS;
+                    if (c < ctot) z[c] = v[u];
                 }
             }
         }
         __syncthreads();
-        // FUSE: the previous unit's stage on the first FUSE_WARPS warps, which then join this
-        // unit's rows, claimed a warp's row block at a time, so the stage hides behind the rows
+        // FUSE: the previous piece's stage on the first FUSE_WARPS warps, which then join this
+        // piece's rows, claimed a warp's row block at a time, so the stage hides behind the rows
         if (FUSE && prev_ne > 0 && warp < FUSE_WARPS) fused_stage<FUSE>(ode, stage, prev_e0, prev_ne, 32 * FUSE_WARPS);
         prev_ne = 0;
         if (rows_on) {
-            // ---- rows: lanes split into groups of lpr (>= UY_RPW) per UY_RPW-row block, so
-            //      that short rows still keep every lane busy
+            // ---- rows: lanes split into groups of lpr per UY_RPW-row block, so that short rows
+            //      still keep every lane busy (lpr, and with it each row's sum, is the same for
+            //      1, 2 and 4 rows per pass)
             const int nvec = tk.cpad_d / Vec<TD>::N + tk.cpad / Vec<TL>::N;
             int lpr = 32;
-            while (lpr > UY_RPW && 2 * nvec <= lpr) lpr >>= 1;
+            while (lpr > UyShape<UY_RPW>::min_lanes && 2 * nvec <= lpr) lpr >>= 1;
             const int gpw = 32 / lpr, g = lane / lpr, sl = lane - g * lpr;
             const int wstep = gpw * UY_RPW;   // rows of one warp's block
             auto claim_rows = [&]() {
@@ -381,7 +397,7 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
             }
         }
         __syncthreads();
-        if (FUSE) {   // the unit's elements (a skipped model's too: the stage decides)
+        if (FUSE) {   // the piece's elements (a skipped model's too: the stage decides)
             prev_e0 = (int)(tk.out_off / ode.nout);
             prev_ne = tk.rows / ode.nout;
         }
@@ -904,29 +920,41 @@ int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 
 struct GemvCfg {
     hbi_handle *h;
-    int smem1, smem2, smax;
+    int smem1, smem2;
     template <typename TD, typename TL> hbi_status operator()() {
         // The limit is a property of the kernel, shared by every handle: only ever raise
         // it, so that building a handle with smaller panels cannot invalidate another's.
         cudaFuncAttributes fa;
         // rows per pass 4 / 8, each plain and with a Cash-Karp stage of either law inside
         // (same grid: the smallest of the occupancies)
-        const void *fns[2][3] = {{(const void *)uy_gemv_kernel<TD, TL, 4, 0>, (const void *)uy_gemv_kernel<TD, TL, 4, 1>,
+        const void *fns[4][3] = {{(const void *)uy_gemv_kernel<TD, TL, 1, 0>, (const void *)uy_gemv_kernel<TD, TL, 1, 1>,
+                                  (const void *)uy_gemv_kernel<TD, TL, 1, 2>},
+                                 {(const void *)uy_gemv_kernel<TD, TL, 2, 0>, (const void *)uy_gemv_kernel<TD, TL, 2, 1>,
+                                  (const void *)uy_gemv_kernel<TD, TL, 2, 2>},
+                                 {(const void *)uy_gemv_kernel<TD, TL, 4, 0>, (const void *)uy_gemv_kernel<TD, TL, 4, 1>,
                                   (const void *)uy_gemv_kernel<TD, TL, 4, 2>},
                                  {(const void *)uy_gemv_kernel<TD, TL, 8, 0>, (const void *)uy_gemv_kernel<TD, TL, 8, 1>,
                                   (const void *)uy_gemv_kernel<TD, TL, 8, 2>}};
-        for (int v = 0; v < 2; ++v) {
-            int occ = 1 << 30;
+        // the occupancy of a row variant (the smallest over its three kernels)
+        auto occupancy = [&](int v, int smem, int &occ) -> hbi_status {
+            occ = 1 << 30;
             for (int f = 0; f < 3; ++f) {
                 HBI_CUDA_TRY(cudaFuncGetAttributes(&fa, fns[v][f]));
-                if (smem2 > fa.maxDynamicSharedSizeBytes)
-                    HBI_CUDA_TRY(cudaFuncSetAttribute(fns[v][f], cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
+                if (smem > fa.maxDynamicSharedSizeBytes)
+                    HBI_CUDA_TRY(cudaFuncSetAttribute(fns[v][f], cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
                 int b = 0;
-                HBI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fns[v][f], GEMV_THREADS, smem2));
-                occ = std::min(occ, b);
+                HBI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fns[v][f], GEMV_THREADS, smem));
+                occ = std::min(occ, std::max(1, b));
             }
-            h->uy_occ[v] = std::max(1, occ);
-        }
+            return HBI_OK;
+        };
+        hbi_status st;
+        int occ[4];
+        for (int v = 0; v < 4; ++v)
+            if ((st = occupancy(v, smem2, occ[v]))) return st;
+        h->smem2 = smem2;
+        h->uy_occ[0] = std::min(occ[0], std::min(occ[1], occ[2]));
+        h->uy_occ[1] = occ[3];
         const void *fvt = (const void *)vt_stream_kernel<TL>;
         HBI_CUDA_TRY(cudaFuncGetAttributes(&fa, fvt));
         if (smem1 > fa.maxDynamicSharedSizeBytes)
@@ -937,7 +965,6 @@ struct GemvCfg {
             set_error("VT stage ring does not fit one SM");
             return HBI_ERR_INVALID_ARG;
         }
-        h->uy_rpw = 4;
         h->vt_pass_cost = VT_PASS_COST;
         set_uy_grid(h, h->uy_occ[0]);
         return HBI_OK;
@@ -974,7 +1001,6 @@ template <typename F> hbi_status dispatch_storage(int storage, F &&f) {
 }
 
 hbi_status gemv_config(hbi_handle *h, int smem1, int smem2) {
-    const int smax = std::max(smem1, smem2);
     if (smem2 > 220 * 1024) {
         set_error("a leaf row unit needs more than 220 KB of gathered input");
         return HBI_ERR_INVALID_ARG;
@@ -982,11 +1008,10 @@ hbi_status gemv_config(hbi_handle *h, int smem1, int smem2) {
     int dev = 0;
     HBI_CUDA_TRY(cudaGetDevice(&dev));
     HBI_CUDA_TRY(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev));
-    GemvCfg cfg{h, smem1, smem2, smax};
+    GemvCfg cfg{h, smem1, smem2};
     hbi_status st = dispatch_storage(h->storage, cfg);
     if (st) return st;
     h->smem1 = smem1;
-    h->smem2 = smem2;
     return HBI_OK;
 }
 
@@ -1354,18 +1379,26 @@ hbi_status pack_operator(hbi_handle *h, const Tree *, std::vector<Block> &blocks
     if ((st = dispatch_storage(h->storage, pk))) return st;
     HBI_CUDA_TRY(cudaDeviceSynchronize());
 
-    // ---- UY tasks sorted by decreasing size for the dynamic scheduler (LPT)
+    // ---- UY tasks for the dynamic scheduler: units by decreasing size, cut by rows
     auto work = [&](const GemvTask &a) { return (int64_t)a.rows * ((int64_t)a.cpad * esl + (int64_t)a.cpad_d * esd); };
     auto bigger = [&](const GemvTask &a, const GemvTask &b) {
         const int64_t ca = work(a), cb = work(b);
         return ca > cb || (ca == cb && (a.data_off < b.data_off || (a.data_off == b.data_off && a.data_off_d < b.data_off_d)));
     };
     std::stable_sort(t2.begin(), t2.end(), bigger);
+    const std::vector<GemvTask> units = t2;
+    t2 = cut_uy_units(units, nout, (int)esl, (int)esd, h->num_sms, UyShape<4>::blocks);
+    std::stable_sort(t2.begin(), t2.end(), bigger);
     h->grid1 = G;
-    int smem1 = (int)(VT_STAGES * VT_STAGE_BYTES), smem2 = 16;
-    for (auto &T : t2) smem2 = std::max<int>(smem2, (int)((T.cpad + T.cpad_d) * acc_bytes));
+    int smem1 = (int)(VT_STAGES * VT_STAGE_BYTES), smem2 = 16, max_rows = 1;
+    for (auto &T : t2) {
+        smem2 = std::max<int>(smem2, (int)((T.cpad + T.cpad_d) * acc_bytes));
+        max_rows = std::max(max_rows, T.rows);
+    }
+    h->uy_rpw = h->uy_rpw_base = max_rows <= 8 ? 1 : (max_rows <= 16 ? 2 : 4);
     // every access of the two product kernels stays inside its buffers (the bounds-checked
-    // build checks the same limits on the device)
+    // build checks the same limits on the device); a piece lies inside its unit and shares its
+    // gather list
     {
         TableLimits L;
         L.n_data1 = d1; L.n_data2 = d2; L.n_data3 = d3;
@@ -1375,7 +1408,7 @@ hbi_status pack_operator(hbi_handle *h, const Tree *, std::vector<Block> &blocks
         L.vt_panel_bytes = (int)VT_PANEL_BYTES; L.vt_x_bytes = (int)VT_X_BYTES; L.vt_max_sub = VT_MAX_SUB;
         L.vt_split_rows = VT_MC_ROWS;
         std::string first;
-        if (check_vt_tables(batches, items, L, &first) + check_uy_tables(t2, gidx, L, &first) > 0) {
+        if (check_vt_tables(batches, items, L, &first) + check_uy_tables(units, gidx, L, &first) > 0) {
             set_error("internal error: an HMVM work table exceeds its buffers (" + first + ")");
             return HBI_ERR_INVALID_ARG;
         }
@@ -1497,15 +1530,16 @@ hbi_status hmvm_run(hbi_handle *h, int phase, typename Vec<TL>::A *xt, typename 
         h->d_tasks2, h->n_tasks2, (const TD *)h->d_data3, (const TL *)h->d_data2, h->d_gidx, h->d_gscale, xt, yp,    \
         counters, d_stop, d_mskip, oa, stage)
         const int f = fuse == nullptr ? 0 : (law == 2 ? 2 : 1);
-        if (h->uy_rpw == 8) {
-            if (f == 2) HBI_UY_LAUNCH(8, 2);
-            else if (f == 1) HBI_UY_LAUNCH(8, 1);
-            else HBI_UY_LAUNCH(8, 0);
-        } else {
-            if (f == 2) HBI_UY_LAUNCH(4, 2);
-            else if (f == 1) HBI_UY_LAUNCH(4, 1);
-            else HBI_UY_LAUNCH(4, 0);
-        }
+        auto rows_per_pass = [&](auto rc) {
+            constexpr int R = decltype(rc)::value;
+            if (f == 2) HBI_UY_LAUNCH(R, 2);
+            else if (f == 1) HBI_UY_LAUNCH(R, 1);
+            else HBI_UY_LAUNCH(R, 0);
+        };
+        if (h->uy_rpw == 8) rows_per_pass(std::integral_constant<int, 8>());
+        else if (h->uy_rpw == 4) rows_per_pass(std::integral_constant<int, 4>());
+        else if (h->uy_rpw == 2) rows_per_pass(std::integral_constant<int, 2>());
+        else rows_per_pass(std::integral_constant<int, 1>());
 #undef HBI_UY_LAUNCH
     }
     HBI_CUDA_TRY(cudaGetLastError());

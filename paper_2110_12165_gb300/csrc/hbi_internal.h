@@ -99,7 +99,7 @@ std::vector<Block> build_partition(const Tree &T, int nin, int nout, double eta,
                                    std::vector<int> *lattice_ij = nullptr);
 
 // ------------------------------------------------------------ HMVM layout
-// One UY-phase work item (a leaf row unit): `rows` outputs, each the dot product of a stored
+// One UY-phase work item (a leaf row unit or a piece of one): `rows` outputs, each the dot product of a stored
 // row with an input vector gathered into shared memory.  A row has two segments: dense
 // near-field columns (element type of the dense stream) followed by low-rank U columns
 // (element type of the factor stream).  Both segments are row-major, 16-byte aligned and
@@ -210,7 +210,8 @@ struct hbi_handle {
     int smem1 = 0, smem2 = 0;               // dynamic shared memory of the two phases
     int grid1 = 0, grid2 = 0;
     // launch configuration (defaults from the build; hbi_autotune may change them)
-    int uy_rpw = 4;                         // UY rows per lane group and pass: 4 or 8
+    int uy_rpw = 4;                         // UY rows per lane group and pass: uy_rpw_base or 8
+    int uy_rpw_base = 4;                    // 1, 2 or 4: the most that leave no warp of a piece without rows
     int uy_occ[2] = {1, 1};                 // UY CTAs per SM that fit, for 4 / 8 rows per pass
     int uy_ctas_per_sm = 1;
     int vt_pass_cost = 8;                   // per-pass cost in the VT per-item shape choice

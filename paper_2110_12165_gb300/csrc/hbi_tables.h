@@ -7,6 +7,7 @@
 
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -101,6 +102,46 @@ int64_t check_uy_tables(const std::vector<Task> &tasks, const std::vector<int> &
         }
     }
     return bad;
+}
+
+// The UY tasks of leaf row units given by decreasing work: each unit cut by rows into pieces of
+// whole elements (nout rows each), which share the unit's gather list.  A piece holds at most the
+// work left (its own unit's included) / (2 x CTA slots), as in guided self-scheduling: with one unit
+// per task the 475 units of a 20,022-element fault leave most of 760 slots idle in one uneven
+// wave (UY phase 68 us uncut, 59 us cut on a GB300; 243 units in FP64 190 against 126 us; 124
+// units 33.5 against 16.5 us), and at 160,000 elements the small last pieces even out the CTAs'
+// ends (475 against 471 us).  A piece gathers its whole input again, so it keeps 24 rows (12
+// rows: 63 us at 20,022 elements) and 112 KB (units of 134 KB cut in two: 46.0 against 44.5 us),
+// unless the pieces would then not fill the slots once: down to 8 rows (2,048 elements with one
+// output each: 12.8 against 16.9 us).
+template <typename Task>
+std::vector<Task> cut_uy_units(const std::vector<Task> &units, int nout, int es_u, int es_d, int sms, int ctas_per_sm) {
+    auto work = [&](const Task &t) { return (int64_t)t.rows * ((int64_t)t.cpad * es_u + (int64_t)t.cpad_d * es_d); };
+    int64_t left = 0, rows = 0;
+    for (const Task &t : units) {
+        left += work(t);
+        rows += t.rows;
+    }
+    const int64_t slots = std::max<int64_t>(1, (int64_t)sms * ctas_per_sm);
+    const int64_t min_rows = std::min<int64_t>(24, std::max<int64_t>(8, (rows + slots - 1) / slots));
+    const int64_t min_elems = (min_rows + nout - 1) / nout, min_work = std::min<int64_t>(112 << 10, left / slots);
+    std::vector<Task> cut;
+    for (const Task &t : units) {
+        const int64_t w = work(t), ne = t.rows / nout, target = std::max<int64_t>(1, left / (2 * slots));
+        const int64_t most = std::min(ne / min_elems, w / std::max<int64_t>(1, min_work));
+        const int64_t np = std::max<int64_t>(1, std::min((w + target - 1) / target, most));
+        for (int64_t q = 0; q < np; ++q) {
+            const int64_t r0 = ne * q / np * nout, r1 = ne * (q + 1) / np * nout;
+            Task c = t;
+            c.rows = (int)(r1 - r0);
+            c.out_off += r0;
+            c.data_off += r0 * t.cpad;
+            c.data_off_d += r0 * t.cpad_d;
+            cut.push_back(c);
+        }
+        left -= w;
+    }
+    return cut;
 }
 
 }  // namespace hbi
