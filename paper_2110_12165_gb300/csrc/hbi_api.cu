@@ -168,7 +168,7 @@ hbi_status run_steps(hbi_handle *h, const hbi_friction *f, double *d_state, doub
         ++batches;
         // the outputs, in case this batch completed every model (rewritten after a further
         // batch; the caller's state is read only at the start), then one host round trip for
-        // the control blocks and the error flag of the bounded device waits
+        // the control blocks
         if ((st = ode_state_out(h, d_state, s, vec))) return st;
         HBI_CUDA_TRY(cudaMemcpy2DAsync(d_t, sizeof(double), &h->d_ctl->t, sizeof(StepCtl), sizeof(double), nm,
                                        cudaMemcpyDeviceToDevice, s));
@@ -176,13 +176,8 @@ hbi_status run_steps(hbi_handle *h, const hbi_friction *f, double *d_state, doub
                                        cudaMemcpyDeviceToDevice, s));
         HBI_CUDA_TRY(cudaMemcpyAsync(h->h_ctl, h->d_ctl, nm * sizeof(StepCtl), cudaMemcpyDeviceToHost, s));
         HBI_CUDA_TRY(cudaMemcpyAsync(h->h_gctl, h->d_gctl, sizeof(GlobalCtl), cudaMemcpyDeviceToHost, s));
-        HBI_CUDA_TRY(cudaMemcpyAsync(h->h_flag, h->d_counters + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
         HBI_CUDA_TRY(cudaStreamSynchronize(s));
-        if (*h->h_flag) {
-            HBI_CUDA_TRY(cudaMemset(h->d_counters + 1, 0, sizeof(int)));
-            set_error("an HMVM stage wait timed out");
-            return HBI_ERR_TIMEOUT;
-        }
+        if ((st = hmvm_check(h))) return st;
         if (h->h_gctl->stop) break;
         if (launched >= max_attempts) { set_error("adaptive stepping did not finish"); return HBI_ERR_TIMEOUT; }
         // the slowest active model sets the next batch: its remaining steps plus as many again
@@ -604,8 +599,7 @@ hbi_status hbi_matvec_async(hbi_handle *h, const double *d_x, double *d_y, hbi_s
     if (!h || !d_x || !d_y) { set_error("handle, x and y are required"); return HBI_ERR_INVALID_ARG; }
     cudaStream_t s = (cudaStream_t)stream;
     hbi_status st = permute_x_in(h, d_x, s);
-    if (!st) st = hmvm_launch(h, s, nullptr);
-    if (!st) st = permute_y_out(h, d_y, s);
+    if (!st) st = hmvm_launch(h, s, nullptr, nullptr, nullptr, nullptr, 0, 1, d_y);
     return st;
 }
 

@@ -61,6 +61,11 @@ constexpr int VT_CW = 8;                     // consumer warps of the VT kernel
 constexpr int VT_THREADS = 32 * (VT_CW + 1); // + one producer warp
 constexpr int VT_MC_ROWS = VT_CW * GEMV_RPW; // rows of a row block split into column chunks
 constexpr int VT_MAX_SUB = 8;                // items per stage batch (<= 32, one producer lane each)
+#ifdef HBI_BOUNDS_CHECK
+constexpr int VT_AHEAD = 0;
+#else
+constexpr int VT_AHEAD = VT_STAGES;          // batches whose panels are copied before the inputs are ready
+#endif
 
 // -------------------------------------------------------- vector decoding
 __device__ __forceinline__ uint4 ld_stream(const void *p) {
@@ -269,9 +274,9 @@ __device__ __forceinline__ void fused_stage(const OdeArgs &A, int stage, int e0,
 template <typename TD, typename TL, int UY_RPW, int FUSE>
 __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv_kernel(
     const GemvTask *__restrict__ tasks, int ntasks, const TD *__restrict__ data_d, const TL *__restrict__ data_l,
-    const int *__restrict__ gidx, const float *__restrict__ gscale, const typename Vec<TL>::A *__restrict__ xt,
-    typename Vec<TL>::A *y, int *counter, const int *stop, const int *__restrict__ mskip, const OdeArgs ode,
-    int stage) {
+    const int *__restrict__ gidx, const float *__restrict__ gscale, const typename Vec<TL>::A *xt,
+    typename Vec<TL>::A *y, int *counter, const int *stop, const int *mskip, double *y_out,
+    const int *__restrict__ perm, const OdeArgs ode, int stage) {
     using A = typename Vec<TL>::A;
     static_assert(std::is_same<typename Vec<TD>::A, A>::value, "segments must share the accumulator");
     constexpr int GU = 4;   // gather: independent index -> value chains per thread
@@ -279,26 +284,19 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
     A *const z = reinterpret_cast<A *>(smem_raw);
     __shared__ int s_next;          // the claimed piece
     __shared__ int s_rowctr;        // FUSE: the piece's next row block (claimed by warps)
-    if (stop != nullptr && *(volatile const int *)stop) {
-        // a skipped product (every active model rejected: k_0 kept) still forms the stage
-        // inputs of the new step size; once every model stopped there is nothing to do
-        if (FUSE && stage < 5 && !*(volatile const int *)&ode.g->stop)
-            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ode.n; i += gridDim.x * blockDim.x) {
-                if (FUSE == 2) stage_vec_elem(ode, stage, i);
-                else stage_elem(ode, stage, i);
-            }
-        return;
-    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = GEMV_THREADS / 32;
     int prev_e0 = 0, prev_ne = 0;   // FUSE: the piece whose rows this CTA wrote last
-    for (;;) {
-        if (threadIdx.x == 0) {
-            s_next = atomicAdd(counter, 1);
-            if (FUSE) s_rowctr = 0;
+    // the first piece is the CTA's own, so that its record and gather indices load while the
+    // kernel before is still running; the others are claimed from the counter
+    for (int ti = blockIdx.x, first = 1;; first = 0) {
+        if (!first) {
+            if (threadIdx.x == 0) s_next = (int)gridDim.x + atomicAdd(counter, 1);
+            __syncthreads();
+            ti = s_next;
         }
-        __syncthreads();
-        const int ti = s_next;
+        if (FUSE && threadIdx.x == 0) s_rowctr = 0;
         if (ti >= ntasks) {
+            if (first) pdl_wait();
             if (FUSE && prev_ne > 0) fused_stage<FUSE>(ode, stage, prev_e0, prev_ne, blockDim.x);
             // every CTA has made its last claim once all have counted themselves out here:
             // the last one rearms the work counter (counter[0]) and this count (counter[2])
@@ -312,7 +310,7 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
             break;
         }
         const GemvTask tk = tasks[ti];
-        bool rows_on = mskip == nullptr || !mskip[tk.model];   // rows of a finished model: nothing to do
+        bool task_ok = true;
 #ifdef HBI_BOUNDS_CHECK
         const bool task_bad =
             threadIdx.x == 0 &&
@@ -322,25 +320,43 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
                    tk.out_off + tk.rows <= g_lim.n_y && tk.gather_off >= 0 &&
                    tk.gather_off + tk.cpad + tk.cpad_d <= g_lim.n_gather &&
                    (int64_t)(tk.cpad + tk.cpad_d) * (int64_t)sizeof(A) <= g_lim.smem_uy);
-        rows_on = rows_on && !__syncthreads_or(task_bad);
+        task_ok = !__syncthreads_or(task_bad);
 #endif
-        if (rows_on) {
-            const int ctot = tk.cpad_d + tk.cpad;
-            // ---- input gather into shared memory: [dense segment | low-rank segment]
-            const int *gi = gidx + tk.gather_off;
-            const float *gs = gscale != nullptr ? gscale + tk.gather_off : nullptr;
-            for (int c0 = threadIdx.x; c0 < ctot; c0 += GU * GEMV_THREADS) {
-                int idx[GU];
+        // ---- input gather into shared memory: [dense segment | low-rank segment]
+        const int ctot = task_ok ? tk.cpad_d + tk.cpad : 0;
+        const int *gi = gidx + tk.gather_off;
+        int idx[GU];
+        auto load_idx = [&](int c0) {
 #pragma unroll
-                for (int u = 0; u < GU; ++u) {
-                    const int c = c0 + u * GEMV_THREADS;
-                    idx[u] = c < ctot ? gi[c] : -1;
+            for (int u = 0; u < GU; ++u) {
+                const int c = c0 + u * GEMV_THREADS;
+                idx[u] = c < ctot ? gi[c] : -1;
 #ifdef HBI_BOUNDS_CHECK
-                    if (HBI_BC(idx[u] == -1 || (idx[u] >= 0 && idx[u] < g_lim.n_xt) ||
-                               (idx[u] <= -2 && -1 - (int64_t)idx[u] < g_lim.n_xt)))
-                        idx[u] = -1;
+                if (HBI_BC(idx[u] == -1 || (idx[u] >= 0 && idx[u] < g_lim.n_xt) ||
+                           (idx[u] <= -2 && -1 - (int64_t)idx[u] < g_lim.n_xt)))
+                    idx[u] = -1;
 #endif
-                }
+            }
+        };
+        load_idx(threadIdx.x);
+        if (first) {
+            pdl_wait();
+            if (stop != nullptr && *(volatile const int *)stop) {
+                // a skipped product (every active model rejected: k_0 kept) still forms the
+                // stage inputs of the new step size; once every model stopped there is nothing
+                // to do
+                if (FUSE && stage < 5 && !*(volatile const int *)&ode.g->stop)
+                    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ode.n; i += gridDim.x * blockDim.x) {
+                        if (FUSE == 2) stage_vec_elem(ode, stage, i);
+                        else stage_elem(ode, stage, i);
+                    }
+                return;
+            }
+        }
+        const bool rows_on = task_ok && (mskip == nullptr || !mskip[tk.model]);   // rows of a finished model: nothing to do
+        if (rows_on) {
+            const float *gs = gscale != nullptr ? gscale + tk.gather_off : nullptr;
+            for (int c0 = threadIdx.x; c0 < ctot;) {
                 A v[GU];
 #pragma unroll
                 for (int u = 0; u < GU; ++u)   // -1: padding; <= -2: the pair at -2 - idx
@@ -357,6 +373,8 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
                     const int c = c0 + u * GEMV_THREADS;
                     if (c < ctot) z[c] = v[u];
                 }
+                c0 += GU * GEMV_THREADS;
+                if (c0 < ctot) load_idx(c0);
             }
         }
         __syncthreads();
@@ -393,7 +411,14 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
                                             lpr, acc);
                 int row;
                 const A v = reduce_scatter<UY_RPW>(acc, sl, lpr, row);
-                if ((sl & (lpr / UY_RPW - 1)) == 0 && row < nr) y[tk.out_off + r0 + row] = v;
+                if ((sl & (lpr / UY_RPW - 1)) == 0 && row < nr) {
+                    if (!FUSE && y_out != nullptr) {   // the caller's order, component-major
+                        const int e_rows = (int)tk.out_off + r0 + row, p = e_rows / ode.nout;
+                        y_out[(size_t)(e_rows - p * ode.nout) * ode.n + perm[p]] = (double)v;
+                    } else {
+                        y[tk.out_off + r0 + row] = v;
+                    }
+                }
             }
         }
         __syncthreads();
@@ -424,6 +449,10 @@ __device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
 __device__ __forceinline__ void mbar_fence_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, unsigned bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+// bytes to come in the current phase, without an arrival
+__device__ __forceinline__ void mbar_add_tx(uint64_t *bar, unsigned bytes) {
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -617,14 +646,13 @@ template <typename TL>
 __global__ void __launch_bounds__(VT_THREADS, VT_CTAS_PER_SM) vt_stream_kernel(
     const VtBatch *__restrict__ batches, const VtItem *__restrict__ items, const int *__restrict__ cta_begin,
     const TL *__restrict__ data, const float *__restrict__ rowscale, typename Vec<TL>::A *xt, const int *stop,
-    int *err, int pass_cost, const int *__restrict__ mskip) {
+    int *err, int pass_cost, const int *mskip) {
     using A = typename Vec<TL>::A;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full[VT_STAGES], empty[VT_STAGES];
     __shared__ VtItem desc[VT_STAGES][VT_MAX_SUB];
     __shared__ int nsub[VT_STAGES];
     __shared__ int s_fail;
-    if (stop != nullptr && *(volatile const int *)stop) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int beg = cta_begin[blockIdx.x], n = cta_begin[blockIdx.x + 1] - beg;
     volatile int *fail = &s_fail;
@@ -643,6 +671,7 @@ __global__ void __launch_bounds__(VT_THREADS, VT_CTAS_PER_SM) vt_stream_kernel(
         // ---- producer warp: batch i into stage i % VT_STAGES once its previous use is
         // released; lane k handles the descriptor and x slice of the batch's item k
         int i = 0;
+        bool stopped;
 #ifndef HBI_BOUNDS_CHECK
         // descriptors ahead of their use: the batch records two batches ahead, the items of
         // the next batch one ahead (the bounds-checked build reads each only once it is checked)
@@ -651,7 +680,32 @@ __global__ void __launch_bounds__(VT_THREADS, VT_CTAS_PER_SM) vt_stream_kernel(
         if (n > 0) b_cur = batches[beg];
         if (n > 1) b_next = batches[beg + 1];
         if (n > 0 && lane < b_cur.nitems) it_cur = items[b_cur.item0 + lane];
+        // the first panels, which depend on the operator alone, before the inputs are ready: the
+        // stage's phase stays open until its x slices are announced below
+        static_assert(VT_STAGES == 2, "one panel from each of the two batch records held");
+        if (lane == 0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            for (int s = 0; s < min(n, VT_STAGES); ++s) {
+                const VtBatch &b = s == 0 ? b_cur : b_next;
+                mbar_add_tx(&full[s], (unsigned)b.pbytes);
+                bulk_g2s(stage_panel(s), data + b.data_off, (unsigned)b.pbytes, &full[s]);
+            }
+        }
+        __syncwarp();
+        pdl_wait();
+        stopped = stop != nullptr && *(volatile const int *)stop;
+        if (stopped && lane == 0) {   // the panels must land before the CTA may exit
+            volatile int never = 0;
+            for (int s = 0; s < min(n, VT_STAGES); ++s) {
+                mbar_arrive(&full[s]);
+                if (!thread_wait(&full[s], 0u, &never)) *fail = 1;
+            }
+        }
+#else
+        pdl_wait();
+        stopped = stop != nullptr && *(volatile const int *)stop;
 #endif
+        if (stopped) return;
         for (; i < n; ++i) {
             const int s = i % VT_STAGES;
 #ifndef HBI_BOUNDS_CHECK
@@ -704,10 +758,11 @@ __global__ void __launch_bounds__(VT_THREADS, VT_CTAS_PER_SM) vt_stream_kernel(
             __syncwarp();
             if (lane == 0) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                mbar_expect_tx(&full[s], (unsigned)(b.pbytes + b.xbytes));
+                mbar_expect_tx(&full[s], (unsigned)(i < VT_AHEAD ? b.xbytes : b.pbytes + b.xbytes));
             }
             __syncwarp();
-            if (lane == 0) bulk_g2s(stage_panel(s), data + b.data_off, (unsigned)b.pbytes, &full[s]);
+            if (lane == 0 && i >= VT_AHEAD)
+                bulk_g2s(stage_panel(s), data + b.data_off, (unsigned)b.pbytes, &full[s]);
             if (lane < b.nitems)
                 bulk_g2s(stage_x(s) + it.zoff, xt + it.x_off, (unsigned)(it.cpad * (int)sizeof(A)), &full[s]);
         }
@@ -720,6 +775,8 @@ __global__ void __launch_bounds__(VT_THREADS, VT_CTAS_PER_SM) vt_stream_kernel(
         __syncwarp();
     } else {
         // ---- consumers
+        pdl_wait();
+        if (stop != nullptr && *(volatile const int *)stop) return;
         A macc[GEMV_RPW];   // per-lane running sums of the current split row block
 #pragma unroll
         for (int q = 0; q < GEMV_RPW; ++q) macc[q] = A(0);
@@ -739,7 +796,10 @@ __global__ void __launch_bounds__(VT_THREADS, VT_CTAS_PER_SM) vt_stream_kernel(
         }
     }
     __syncthreads();
-    if (tid == 0 && s_fail) atomicExch(err, 1);
+    if (tid == 0 && s_fail) {   // err may be host memory
+        *(volatile int *)err = 1;
+        __threadfence_system();
+    }
 }
 
 // A wait that can never complete (an mbarrier phase that expects one arrival nobody makes),
@@ -772,19 +832,14 @@ hbi_status stalled_wait_status(cudaStream_t s) {
 }
 
 template <typename A>
-__global__ void permute_in_kernel(const double *__restrict__ x, const int *__restrict__ perm, int n, int nin,
-                                  A *__restrict__ xt) {
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const int e = perm[p];
+__global__ void permute_in_kernel(const double *x, const int *__restrict__ perm, int n, int nin, A *__restrict__ xt) {
+    const int p0 = blockIdx.x * blockDim.x + threadIdx.x;
+    int e = p0 < n ? perm[p0] : 0;
+    pdl_wait();
+    for (int p = p0; p < n;) {
         for (int c = 0; c < nin; ++c) xt[(size_t)nin * p + c] = (A)x[(size_t)c * n + e];
-    }
-}
-template <typename A>
-__global__ void permute_out_kernel(const A *__restrict__ yp, const int *__restrict__ perm, int n, int nout,
-                                   double *__restrict__ y) {
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const int e = perm[p];
-        for (int c = 0; c < nout; ++c) y[(size_t)c * n + e] = (double)yp[(size_t)nout * p + c];
+        p += gridDim.x * blockDim.x;
+        if (p < n) e = perm[p];
     }
 }
 
@@ -1437,6 +1492,8 @@ hbi_status pack_operator(hbi_handle *h, const Tree *, std::vector<Block> &blocks
     HBI_ALLOC_TRY(&h->d_xt2, (ntot_in + tcount + 16) * acc_bytes);
     HBI_CUDA_TRY(cudaMemset(h->d_xt2, 0, (ntot_in + tcount + 16) * acc_bytes));
     HBI_ALLOC_TRY(&h->d_yp, (size_t)nout * n * acc_bytes);
+    HBI_CUDA_TRY(cudaMallocHost((void **)&h->h_flag, sizeof(int)));
+    *h->h_flag = 0;
     HBI_ALLOC_TRY(&h->d_counters, 4 * sizeof(int));
     HBI_CUDA_TRY(cudaMemset(h->d_counters, 0, 4 * sizeof(int)));
 
@@ -1501,48 +1558,48 @@ hbi_status pack_operators(hbi_handle *h, std::vector<Block> &blocks, const std::
 
 // ----------------------------------------------------------------- launch
 namespace {
-// One product with explicit buffers.  phase: -1 = whole product, 0 = VT, 2 = UY (with the
-// reset of its work counter unless reset = false, so that it can also be launched alone and
-// repeatedly); 1 launches nothing (kept so the phase timing keeps its layout).  counters[0] is
-// the UY work counter, counters[1] an error flag that a VT CTA sets when one of its bounded
-// waits gives up (cleared only when it is reported), counters[2] the UY CTAs that finished
-// (the last one sets counters[0] and counters[2] back to zero).
+// One product with explicit buffers.  phase: -1 = whole product, 0 = VT, 2 = UY; 1 launches
+// nothing (kept so the phase timing keeps its layout).  counters[0] is the UY work counter and
+// counters[2] counts the UY CTAs that finished; every UY launch leaves both at zero.  err: the
+// flag that a VT CTA sets when one of its bounded waits gives up.  y_out: see hmvm_launch.
 template <typename TD, typename TL>
-hbi_status hmvm_run(hbi_handle *h, int phase, typename Vec<TL>::A *xt, typename Vec<TL>::A *yp, int *counters,
-                    cudaStream_t s, const int *d_stop, const int *d_mskip = nullptr, bool reset = true,
-                    const OdeArgs *fuse = nullptr, int stage = 0, int law = 1) {
+hbi_status hmvm_run(hbi_handle *h, int phase, typename Vec<TL>::A *xt, typename Vec<TL>::A *yp, int *counters, int *err,
+                    cudaStream_t s, const int *d_stop, const int *d_mskip = nullptr, const OdeArgs *fuse = nullptr,
+                    int stage = 0, int law = 1, double *y_out = nullptr) {
 #ifdef HBI_BOUNDS_CHECK
     // from device memory: a copy captured into the attempt graph stays valid at every replay
     HBI_CUDA_TRY(cudaMemcpyToSymbolAsync(g_lim, h->d_lim, sizeof(DevLimits), 0, cudaMemcpyDeviceToDevice, s));
 #endif
     if (phase <= 0) {
         if (h->n_tasks1)
-            vt_stream_kernel<TL><<<h->grid1, VT_THREADS, h->smem1, s>>>(
-                h->d_batches1, h->d_items1, h->d_vt_begin, (const TL *)h->d_data1, h->d_rowscale, xt, d_stop,
-                counters + 1, h->vt_pass_cost, d_mskip);
+            HBI_CUDA_TRY(launch_dependent(vt_stream_kernel<TL>, h->grid1, VT_THREADS, h->smem1, s, h->d_batches1,
+                                          h->d_items1, h->d_vt_begin, (const TL *)h->d_data1, h->d_rowscale, xt, d_stop,
+                                          err, h->vt_pass_cost, d_mskip));
     }
     if (phase < 0 || phase == 2) {
-        if (reset) HBI_CUDA_TRY(cudaMemsetAsync(counters, 0, sizeof(int), s));
-        const OdeArgs none{};
-        const OdeArgs &oa = fuse != nullptr ? *fuse : none;
-#define HBI_UY_LAUNCH(R, F)                                                                                        \
-    uy_gemv_kernel<TD, TL, R, F><<<h->grid2, GEMV_THREADS, h->smem2, s>>>(                                         \
-        h->d_tasks2, h->n_tasks2, (const TD *)h->d_data3, (const TL *)h->d_data2, h->d_gidx, h->d_gscale, xt, yp,    \
-        counters, d_stop, d_mskip, oa, stage)
+        OdeArgs oa{};
+        if (fuse != nullptr) oa = *fuse;
+        oa.n = h->n;
+        oa.nout = h->nout;
         const int f = fuse == nullptr ? 0 : (law == 2 ? 2 : 1);
-        auto rows_per_pass = [&](auto rc) {
-            constexpr int R = decltype(rc)::value;
-            if (f == 2) HBI_UY_LAUNCH(R, 2);
-            else if (f == 1) HBI_UY_LAUNCH(R, 1);
-            else HBI_UY_LAUNCH(R, 0);
+        auto launch = [&](auto rc, auto fc) {
+            return launch_dependent(uy_gemv_kernel<TD, TL, decltype(rc)::value, decltype(fc)::value>, h->grid2,
+                                    GEMV_THREADS, h->smem2, s, h->d_tasks2, h->n_tasks2, (const TD *)h->d_data3,
+                                    (const TL *)h->d_data2, h->d_gidx, h->d_gscale, xt, yp, counters, d_stop, d_mskip,
+                                    y_out, h->d_perm, oa, stage);
         };
-        if (h->uy_rpw == 8) rows_per_pass(std::integral_constant<int, 8>());
-        else if (h->uy_rpw == 4) rows_per_pass(std::integral_constant<int, 4>());
-        else if (h->uy_rpw == 2) rows_per_pass(std::integral_constant<int, 2>());
-        else rows_per_pass(std::integral_constant<int, 1>());
-#undef HBI_UY_LAUNCH
+        auto rows_per_pass = [&](auto rc) {
+            if (f == 2) return launch(rc, std::integral_constant<int, 2>());
+            if (f == 1) return launch(rc, std::integral_constant<int, 1>());
+            return launch(rc, std::integral_constant<int, 0>());
+        };
+        switch (h->uy_rpw) {
+            case 8: HBI_CUDA_TRY(rows_per_pass(std::integral_constant<int, 8>())); break;
+            case 4: HBI_CUDA_TRY(rows_per_pass(std::integral_constant<int, 4>())); break;
+            case 2: HBI_CUDA_TRY(rows_per_pass(std::integral_constant<int, 2>())); break;
+            default: HBI_CUDA_TRY(rows_per_pass(std::integral_constant<int, 1>())); break;
+        }
     }
-    HBI_CUDA_TRY(cudaGetLastError());
     return HBI_OK;
 }
 struct PhaseRun {
@@ -1550,34 +1607,32 @@ struct PhaseRun {
     int phase;
     cudaStream_t s;
     const int *stop, *mskip;
-    bool reset;
     void *xt = nullptr;
     const OdeArgs *fuse = nullptr;
     int stage = 0;
     int law = 1;
+    double *y_out = nullptr;
     template <typename TD, typename TL> hbi_status operator()() {
         using A = typename Vec<TL>::A;
-        return hmvm_run<TD, TL>(h, phase, (A *)(xt != nullptr ? xt : h->d_xt), (A *)h->d_yp, h->d_counters, s, stop,
-                                mskip, reset, fuse, stage, law);
+        return hmvm_run<TD, TL>(h, phase, (A *)(xt != nullptr ? xt : h->d_xt), (A *)h->d_yp, h->d_counters, h->h_flag, s,
+                                stop, mskip, fuse, stage, law, y_out);
     }
 };
 }  // namespace
 
 hbi_status hmvm_phase(hbi_handle *h, int phase, cudaStream_t s, const int *d_stop) {
-    return dispatch_storage(h->storage, PhaseRun{h, phase, s, d_stop, nullptr, true});
+    return dispatch_storage(h->storage, PhaseRun{h, phase, s, d_stop, nullptr});
 }
 
-hbi_status hmvm_launch(hbi_handle *h, cudaStream_t s, const int *d_stop, const int *d_mskip, bool reset_counter,
-                       void *xt, const OdeArgs *fuse, int stage, int law) {
-    return dispatch_storage(h->storage, PhaseRun{h, -1, s, d_stop, d_mskip, reset_counter, xt, fuse, stage, law});
+hbi_status hmvm_launch(hbi_handle *h, cudaStream_t s, const int *d_stop, const int *d_mskip, void *xt,
+                       const OdeArgs *fuse, int stage, int law, double *y_out) {
+    return dispatch_storage(h->storage, PhaseRun{h, -1, s, d_stop, d_mskip, xt, fuse, stage, law, y_out});
 }
 
 // After the stream is synchronised: HBI_ERR_TIMEOUT if a bounded device wait gave up.
 hbi_status hmvm_check(hbi_handle *h) {
-    int err = 0;
-    HBI_CUDA_TRY(cudaMemcpy(&err, h->d_counters + 1, sizeof(int), cudaMemcpyDeviceToHost));
-    if (err) {
-        HBI_CUDA_TRY(cudaMemset(h->d_counters + 1, 0, sizeof(int)));
+    if (*(volatile int *)h->h_flag) {
+        *h->h_flag = 0;
         set_error("an HMVM stage wait timed out");
         return HBI_ERR_TIMEOUT;
     }
@@ -1587,20 +1642,9 @@ hbi_status hmvm_check(hbi_handle *h) {
 hbi_status permute_x_in(hbi_handle *h, const double *d_x, cudaStream_t s) {
     const int grid = std::max(1, std::min((h->n + 255) / 256, 4 * std::max(1, h->num_sms)));
     if (h->storage == HBI_FP64)
-        permute_in_kernel<double><<<grid, 256, 0, s>>>(d_x, h->d_perm, h->n, h->nin, (double *)h->d_xt);
+        HBI_CUDA_TRY(launch_dependent(permute_in_kernel<double>, grid, 256, 0, s, d_x, h->d_perm, h->n, h->nin, (double *)h->d_xt));
     else
-        permute_in_kernel<float><<<grid, 256, 0, s>>>(d_x, h->d_perm, h->n, h->nin, (float *)h->d_xt);
-    HBI_CUDA_TRY(cudaGetLastError());
-    return HBI_OK;
-}
-
-hbi_status permute_y_out(hbi_handle *h, double *d_y, cudaStream_t s) {
-    const int grid = std::max(1, std::min((h->n + 255) / 256, 4 * std::max(1, h->num_sms)));
-    if (h->storage == HBI_FP64)
-        permute_out_kernel<double><<<grid, 256, 0, s>>>((const double *)h->d_yp, h->d_perm, h->n, h->nout, d_y);
-    else
-        permute_out_kernel<float><<<grid, 256, 0, s>>>((const float *)h->d_yp, h->d_perm, h->n, h->nout, d_y);
-    HBI_CUDA_TRY(cudaGetLastError());
+        HBI_CUDA_TRY(launch_dependent(permute_in_kernel<float>, grid, 256, 0, s, d_x, h->d_perm, h->n, h->nin, (float *)h->d_xt));
     return HBI_OK;
 }
 
@@ -1659,13 +1703,9 @@ struct NoallocRun {
         A *yp = reinterpret_cast<A *>(base + off);
         const int grid = std::max(1, std::min((h->n + 255) / 256, 4 * std::max(1, h->num_sms)));
         HBI_CUDA_TRY(cudaMemsetAsync(xt + nxt, 0, 16 * sizeof(A), s));   // guard elements
-        HBI_CUDA_TRY(cudaMemsetAsync(counters + 1, 0, 2 * sizeof(int), s));   // error flag, UY finish count
-        permute_in_kernel<A><<<grid, 256, 0, s>>>(x, h->d_perm, h->n, h->nin, xt);
-        hbi_status st = hmvm_run<TD, TL>(h, -1, xt, yp, counters, s, nullptr);   // clears the work counter
-        if (st) return st;
-        permute_out_kernel<A><<<grid, 256, 0, s>>>(yp, h->d_perm, h->n, h->nout, y);
-        HBI_CUDA_TRY(cudaGetLastError());
-        return HBI_OK;
+        HBI_CUDA_TRY(cudaMemsetAsync(counters, 0, 3 * sizeof(int), s));   // work counter, error flag, UY finish count
+        HBI_CUDA_TRY(launch_dependent(permute_in_kernel<A>, grid, 256, 0, s, x, h->d_perm, h->n, h->nin, xt));
+        return hmvm_run<TD, TL>(h, -1, xt, yp, counters, counters + 1, s, nullptr, nullptr, nullptr, 0, 1, y);
     }
 };
 }  // namespace

@@ -65,6 +65,38 @@ struct DevScratch {
     }
 };
 
+// ------------------------------------------------------------ dependent launches
+// The kernels of a product (and of an attempt) are launched with programmatic stream
+// serialisation: a kernel may start once every CTA of the one before it has exited, before that
+// kernel's completion is signalled, and reads or writes nothing that an earlier kernel produces
+// or reads before its own pdl_wait(), which returns once the earlier kernels have completed and
+// their writes are visible.  What runs ahead of the wait depends on the operator alone: barriers,
+// task records, gather indices, the first V^T panels.  One product (V^T and UY phase) takes 19.7
+// us at 2,048 elements in FP64 against 22.0 us with plain launches, 20.0 against 22.1 us at 5,246
+// and 75.7 against 78.6 us at 20,022 in mixed storage.  No kernel triggers its successor earlier
+// than at its own end: a UY CTA that becomes resident beside a V^T CTA inherits its shared-memory
+// split, and the 28 KB of L1 left hold too few of UY's loads in flight (N = 160,000: 748 against
+// 630 us).  Not used in the bounds-checked build, which copies its limits between the launches.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+#ifndef HBI_BOUNDS_CHECK
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+#endif
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 // ------------------------------------------------------------ host geometry
 struct Frames {
     // per element (original order): centre, normal, strike, dip
@@ -218,7 +250,7 @@ struct hbi_handle {
     void *d_xt = nullptr;                   // [x (nin N) | t (n_t) | 16 zero guards] in accumulation type
     void *d_xt2 = nullptr;                  // a second one: consecutive products of an attempt alternate
     void *d_yp = nullptr;                   // nout N accumulation type
-    int *d_counters = nullptr;              // [0] UY work counter, [1] error flag of bounded device waits
+    int *d_counters = nullptr;              // [0] UY work counter, [2] UY CTAs that finished
     hbi::TableLimits lim;                   // the buffers the product's work tables index
     void *d_lim = nullptr;                  // bounds-checked build: the same limits on the device
     int64_t bytes_factors = 0, bytes_algorithmic = 0, bytes_alg_vt = 0, bytes_alg_uy = 0;
@@ -244,7 +276,7 @@ struct hbi_handle {
     hbi::GlobalCtl *d_gctl = nullptr;
     int *d_mskip = nullptr;                 // 2 x n_models: models whose first / other stage products are skipped
     hbi::GlobalCtl *h_gctl = nullptr;       // pinned mirror
-    int *h_flag = nullptr;                  // pinned mirror of the bounded-wait error flag
+    int *h_flag = nullptr;                  // error flag of bounded device waits (pinned; the kernels write it)
     hbi_step_record *d_rec = nullptr;       // n_models x rec_cap
     int rec_cap = 0;
     cudaStream_t cap_stream = nullptr;
@@ -279,23 +311,22 @@ hbi_status pack_multi(hbi_handle *h, std::vector<Block> &blocks, const std::vect
 void multi_free(hbi_handle *h);
 // d_stop: the whole product returns at once while *d_stop != 0; d_mskip (optional, one int
 // per model): the rows / columns of model m are skipped while d_mskip[m] != 0.
-// reset_counter = false: leave out the reset of the UY work counter before the launch (every
-// UY launch that runs to its end leaves the counter at zero; used inside the attempt graph).
+// y_out (optional): the UY phase writes the product there in the caller's order, component-major
+// FP64, instead of h->d_yp.
 // xt: the input buffer of the product (nullptr: h->d_xt; the attempt alternates h->d_xt and
 // h->d_xt2).  fuse != nullptr: the UY phase also runs Cash-Karp stage `stage` (0..5, the last
 // with the error maxima) of the law `law` (1 fixed rake, 2 rake-free) for the elements of
 // each leaf row unit as soon as the unit's rows are written, with fuse->xt (the other buffer)
 // receiving the next product's input; with *d_stop set it runs stages 0-4 alone.
 hbi_status hmvm_launch(hbi_handle *h, cudaStream_t s, const int *d_stop, const int *d_mskip = nullptr,
-                       bool reset_counter = true, void *xt = nullptr, const OdeArgs *fuse = nullptr, int stage = 0,
-                       int law = 1);
+                       void *xt = nullptr, const OdeArgs *fuse = nullptr, int stage = 0, int law = 1,
+                       double *y_out = nullptr);
 void set_uy_grid(hbi_handle *h, int per_sm);
 hbi_status hmvm_check(hbi_handle *h);   // after a stream sync: TIMEOUT if a device wait gave up
 hbi_status stalled_wait_status(cudaStream_t s);
 // phases separately (0 = VT, 1 = nothing, 2 = UY), for timing
 hbi_status hmvm_phase(hbi_handle *h, int phase, cudaStream_t s, const int *d_stop);
 hbi_status permute_x_in(hbi_handle *h, const double *d_x, cudaStream_t s);
-hbi_status permute_y_out(hbi_handle *h, double *d_y, cudaStream_t s);
 hbi_status device_build_factors(hbi_handle *h, const Tree &T, std::vector<Block> &blocks,
                                 double eps, std::vector<void *> &owned);
 hbi_status upload_geometry(hbi_handle *h, const double *h_verts, const double *h_rake);

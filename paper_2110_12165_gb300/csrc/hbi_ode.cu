@@ -186,6 +186,7 @@ __global__ void stop_kernel(OdeArgs A) { stop_models(A); }
 // first product input; the CTA that finishes last then runs the step control of every model
 // (Eqs. 14-15, records, next dt) and sets the stop and skip flags, and rearms its counter.
 __global__ void commit_ctl_kernel(OdeArgs A) {
+    pdl_wait();
     if (all_stopped(A)) return;
     __shared__ int s_last;
     const int n = A.n;
@@ -561,7 +562,6 @@ hbi_status ode_alloc(hbi_handle *h, int rec_cap) {
         HBI_ALLOC_TRY(&h->d_gctl, sizeof(GlobalCtl));
         HBI_CUDA_TRY(cudaMemset(h->d_gctl, 0, sizeof(GlobalCtl)));
         HBI_CUDA_TRY(cudaMallocHost(&h->h_gctl, sizeof(GlobalCtl)));
-        HBI_CUDA_TRY(cudaMallocHost(&h->h_flag, sizeof(int)));
         HBI_ALLOC_TRY(&h->d_mskip, 2 * nm * sizeof(int));
         HBI_CUDA_TRY(cudaMemset(h->d_mskip, 0, 2 * nm * sizeof(int)));
         if (!h->d_model) {
@@ -662,11 +662,11 @@ hbi_status ode_attempt(hbi_handle *h, cudaStream_t s, int vec) {
             OdeArgs F = A;
             F.xt = xb[(st + 1) & 1];
             hbi_status r = hmvm_launch(h, s, st == 0 ? &h->d_gctl->skip0 : stop,
-                                       st == 0 ? h->d_mskip : h->d_mskip + h->n_models, false, xb[st & 1], &F, st);
+                                       st == 0 ? h->d_mskip : h->d_mskip + h->n_models, xb[st & 1], &F, st);
             if (r) return r;
         }
-        commit_ctl_kernel<<<g, ODE_BLOCK, 0, s>>>(A);   // controller, commit and stop flags in one launch
-        HBI_CUDA_TRY(cudaGetLastError());
+        // controller, commit and stop flags in one launch
+        HBI_CUDA_TRY(launch_dependent(commit_ctl_kernel, g, ODE_BLOCK, 0, s, A));
         return HBI_OK;
     }
     // rake-free friction: the same, with its stage functions; then controller, commit, stop
@@ -675,7 +675,7 @@ hbi_status ode_attempt(hbi_handle *h, cudaStream_t s, int vec) {
         OdeArgs F = A;
         F.xt = xb[(st + 1) & 1];
         hbi_status r = hmvm_launch(h, s, st == 0 ? &h->d_gctl->skip0 : stop,
-                                   st == 0 ? h->d_mskip : h->d_mskip + h->n_models, false, xb[st & 1], &F, st, 2);
+                                   st == 0 ? h->d_mskip : h->d_mskip + h->n_models, xb[st & 1], &F, st, 2);
         if (r) return r;
     }
     controller_kernel<<<1, 256, 0, s>>>(A);
@@ -702,8 +702,7 @@ hbi_status ode_attempt_profiled(hbi_handle *h, cudaStream_t s, cudaEvent_t *ev, 
     };
     hbi_status r;
     for (int st = 0; st < 6; ++st) {
-        if ((r = hmvm_launch(h, s, st == 0 ? &h->d_gctl->skip0 : stop, st == 0 ? h->d_mskip : h->d_mskip + h->n_models,
-                             false)) ||
+        if ((r = hmvm_launch(h, s, st == 0 ? &h->d_gctl->skip0 : stop, st == 0 ? h->d_mskip : h->d_mskip + h->n_models)) ||
             (r = mark(0)))
             return r;
         if (st < 5) stage_kernel<<<g, ODE_BLOCK, 0, s>>>(A, st);

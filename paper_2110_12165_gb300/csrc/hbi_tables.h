@@ -125,13 +125,16 @@ std::vector<Task> cut_uy_units(const std::vector<Task> &units, int nout, int es_
     const int64_t slots = std::max<int64_t>(1, (int64_t)sms * ctas_per_sm);
     const int64_t min_rows = std::min<int64_t>(24, std::max<int64_t>(8, (rows + slots - 1) / slots));
     const int64_t min_elems = (min_rows + nout - 1) / nout, min_work = std::min<int64_t>(112 << 10, left / slots);
+    const int64_t whole = nout % 2 ? 4 : 2;   // elements of whole 4-row blocks: only a unit's last piece ends in a partial one
     std::vector<Task> cut;
     for (const Task &t : units) {
         const int64_t w = work(t), ne = t.rows / nout, target = std::max<int64_t>(1, left / (2 * slots));
         const int64_t most = std::min(ne / min_elems, w / std::max<int64_t>(1, min_work));
         const int64_t np = std::max<int64_t>(1, std::min((w + target - 1) / target, most));
         for (int64_t q = 0; q < np; ++q) {
-            const int64_t r0 = ne * q / np * nout, r1 = ne * (q + 1) / np * nout;
+            const int64_t r0 = ne * q / np / whole * whole * nout;
+            const int64_t r1 = q + 1 < np ? ne * (q + 1) / np / whole * whole * nout : t.rows;
+            if (r0 == r1) continue;
             Task c = t;
             c.rows = (int)(r1 - r0);
             c.out_off += r0;
