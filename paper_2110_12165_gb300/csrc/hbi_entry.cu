@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(ACA_THREADS) aca_kernel(EntryGeo g, const AcaJ
             continue;
         }
         const double piv = vk[j];
+        __syncthreads();   // every thread holds the pivot before its entry is divided
         for (int J = threadIdx.x; J < nc; J += blockDim.x) vk[J] /= piv;
         // residual column j -> U[:, k]
         double *uk = jb.U + (size_t)k * m;
