@@ -5,12 +5,21 @@
 // them, and their host driver.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "hbi_entry_math.cuh"
 #include "hbi_internal.h"
 
 namespace hbi {
+
+__global__ void edge_const_kernel(EntryGeo g, int n, EdgeConst *out) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n * g.nv) return;
+    const int j = k / g.nv, a = k - j * g.nv, a1 = a + 1 == g.nv ? 0 : a + 1;
+    const double *vj = g.verts + (size_t)j * g.nv * 3;
+    out[k] = edge_const(vj + 3 * a, vj + 3 * a1);
+}
 
 // ---------------------------------------------------------------- dense fill
 struct DenseJob {
@@ -40,13 +49,24 @@ struct AcaJob {
     double *U, *V;        // m x rmax and nc x rmax, column-major
     unsigned char *flags; // m + nc bytes (used rows, used columns)
 };
-struct AcaOut { int rank, status; };  // status: 0 converged, 1 rank budget exhausted, 2 capped, 3 singular
+// status: 0 converged, 1 rank budget exhausted, 2 capped, 3 singular, 4 evaluated whole and some
+// pair singular (which ACA need not meet)
+struct AcaOut { int rank, status; };
 
-constexpr int ACA_THREADS = 256;
-constexpr int ACA_WARPS = ACA_THREADS / 32;
+// The entries are what ACA costs (a pair of elements takes about 2,000 FP64 instructions, and an
+// SM issues one FP64 warp instruction in 16 cycles), so a block gets the CTA that its larger side
+// fills, several of the small ones share an SM, and the largest blocks start first.  A block whose
+// pairs are fewer than ACA_DENSE rows and columns of them is evaluated whole before its ACA: a row
+// or column needs one of the pair's n_out rows or n_in columns but evaluates the pair, and its
+// last warp is mostly idle, so 24 rows and columns of a 40 x 40 block cost twice its 1,600 pairs.
+// With one 256-thread CTA (182 registers, one per SM) for every block, in partition order: 282
+// ms for the 9,086 blocks of a 20,022-element fault; so 170 ms one class
+// after the other, less side by side.
+constexpr int ACA_DENSE = 20;
 
 // block-wide argmax of (value, index) with ties to the smaller index; -1 if all excluded
 __device__ void block_argmax(double v, int idx, double *sv, int *si, double &best, int &bidx) {
+    const int nw = blockDim.x >> 5;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -59,7 +79,7 @@ __device__ void block_argmax(double v, int idx, double *sv, int *si, double &bes
     if (threadIdx.x == 0) {
         double bv = sv[0];
         int bi = si[0];
-        for (int k = 1; k < ACA_WARPS; ++k)
+        for (int k = 1; k < nw; ++k)
             if (si[k] >= 0 && (bi < 0 || sv[k] > bv || (sv[k] == bv && si[k] < bi))) { bv = sv[k]; bi = si[k]; }
         sv[0] = bv; si[0] = bi;
     }
@@ -77,7 +97,7 @@ __device__ double block_sum(double v, double *sv) {
     __syncthreads();
     if (threadIdx.x == 0) {
         double s = 0.0;
-        for (int k = 0; k < ACA_WARPS; ++k) s += sv[k];
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += sv[k];
         sv[0] = s;
     }
     __syncthreads();
@@ -92,20 +112,37 @@ __device__ double block_sum(double v, double *sv) {
 // residual row moves on to the first unused row; stop once |u_k||v_k| <= eps ||S_k||_F
 // (Frobenius norm of the approximant updated recursively).  Reaching the rank cap
 // floor(m n / (m + n)) marks the block for dense storage.
-template <bool HALF>
-__global__ void __launch_bounds__(ACA_THREADS) aca_kernel(EntryGeo g, const AcaJob *jobs, AcaOut *outs,
-                                                          double eps) {
+// FULL: the block's entries are evaluated first, into `full` (row-major, nc columns).
+template <bool HALF, int THREADS, bool FULL>
+__device__ void aca_block(const EntryGeo &g, const AcaJob &jb, AcaOut *out, double eps, double *full) {
+    constexpr int ACA_WARPS = THREADS / 32;
     __shared__ double sv[ACA_WARPS];
     __shared__ int si[ACA_WARPS];
     __shared__ double s_cross[ACA_WARPS];
-    const AcaJob jb = jobs[blockIdx.x];
     const int m = jb.m, nc = jb.nc;
     unsigned char *urow = jb.flags, *ucol = jb.flags + m;
     for (int k = threadIdx.x; k < m + nc; k += blockDim.x) jb.flags[k] = 0;
+    bool singular = false;
+    if (FULL) {
+        const int np = jb.tau_size * jb.sig_size;
+        for (int p = threadIdx.x; p < np; p += blockDim.x) {
+            const int ii = p / jb.sig_size, jj = p - ii * jb.sig_size;
+            double E[3][2];
+            singular |= !pair_op<HALF>(g, jb.tau_start + ii, jb.sig_start + jj, E);
+            for (int a = 0; a < g.nout; ++a)
+                for (int c = 0; c < g.nin; ++c) full[(size_t)(ii * g.nout + a) * nc + jj * g.nin + c] = E[a][c];
+        }
+        if (__syncthreads_or(singular)) {
+            if (threadIdx.x == 0) {
+                out->rank = 0;
+                out->status = 4;
+            }
+            return;
+        }
+    }
     __syncthreads();
     int k = 0, i = 0, status = 0;
     double normS2 = 0.0;
-    bool singular = false;
     for (int guard = 0; guard < m + nc + 2; ++guard) {
         if (k >= jb.rcap) { status = 2; break; }
         if (k >= jb.rmax) { status = 1; break; }
@@ -115,10 +152,10 @@ __global__ void __launch_bounds__(ACA_THREADS) aca_kernel(EntryGeo g, const AcaJ
             const int ie = jb.tau_start + i / g.nout, co = i % g.nout;
             for (int jj = threadIdx.x; jj < jb.sig_size; jj += blockDim.x) {
                 double E[3][2];
-                if (!pair_op<HALF>(g, ie, jb.sig_start + jj, E)) singular = true;
+                if (!FULL && !pair_op<HALF>(g, ie, jb.sig_start + jj, E)) singular = true;
                 for (int c = 0; c < g.nin; ++c) {
                     const int J = jj * g.nin + c;
-                    double val = E[co][c];
+                    double val = FULL ? full[(size_t)i * nc + J] : E[co][c];
                     for (int l = 0; l < k; ++l) val -= jb.U[(size_t)l * m + i] * jb.V[(size_t)l * nc + J];
                     vk[J] = val;
                 }
@@ -161,10 +198,10 @@ __global__ void __launch_bounds__(ACA_THREADS) aca_kernel(EntryGeo g, const AcaJ
             const int je = jb.sig_start + j / g.nin, ci = j % g.nin;
             for (int ii = threadIdx.x; ii < jb.tau_size; ii += blockDim.x) {
                 double E[3][2];
-                if (!pair_op<HALF>(g, jb.tau_start + ii, je, E)) singular = true;
+                if (!FULL && !pair_op<HALF>(g, jb.tau_start + ii, je, E)) singular = true;
                 for (int a = 0; a < g.nout; ++a) {
                     const int I = ii * g.nout + a;
-                    double val = E[a][ci];
+                    double val = FULL ? full[(size_t)I * nc + j] : E[a][ci];
                     for (int l = 0; l < k; ++l) val -= jb.V[(size_t)l * nc + j] * jb.U[(size_t)l * m + I];
                     uk[I] = val;
                 }
@@ -217,14 +254,26 @@ __global__ void __launch_bounds__(ACA_THREADS) aca_kernel(EntryGeo g, const AcaJ
         i = nxt;
     }
     // reduce the singular flag
-    __shared__ int s_sing;
-    if (threadIdx.x == 0) s_sing = 0;
-    __syncthreads();
-    if (singular) atomicOr(&s_sing, 1);
-    __syncthreads();
+    const int sing = __syncthreads_or(singular);
     if (threadIdx.x == 0) {
-        outs[blockIdx.x].rank = k;
-        outs[blockIdx.x].status = s_sing ? 3 : status;
+        out->rank = k;
+        out->status = sing ? 3 : status;
+    }
+}
+
+template <bool HALF, int THREADS>
+__global__ void __launch_bounds__(THREADS) aca_kernel(EntryGeo g, const AcaJob *jobs, AcaOut *outs, double eps) {
+    aca_block<HALF, THREADS, false>(g, jobs[blockIdx.x], outs + blockIdx.x, eps, nullptr);
+}
+
+// Small blocks, evaluated whole: persistent CTAs, each with one slot of `slot` doubles of scratch
+// (all of them together stay in L2).
+template <bool HALF, int THREADS>
+__global__ void __launch_bounds__(THREADS) aca_full_kernel(EntryGeo g, const AcaJob *jobs, AcaOut *outs, int njobs,
+                                                           double eps, double *scratch, int64_t slot) {
+    for (int b = blockIdx.x; b < njobs; b += gridDim.x) {
+        aca_block<HALF, THREADS, true>(g, jobs[b], outs + b, eps, scratch + blockIdx.x * slot);
+        __syncthreads();
     }
 }
 
@@ -240,17 +289,66 @@ hbi_status dev_alloc(T **p, size_t count, std::vector<void *> &owned) {
     *p = (T *)q;
     return HBI_OK;
 }
+
+// The launch class of a block: 0-2 by the CTA its larger side fills (256, 128, 64 threads), 3
+// evaluated whole
+constexpr int ACA_CLASSES = 4;
+int aca_class(int tau, int sig, bool stepwise) {
+    if (!stepwise && ((int64_t)tau * sig + 31) / 32 <= ACA_DENSE * ((tau + 31) / 32 + (sig + 31) / 32)) return 3;
+    const int side = std::max(tau, sig);
+    return side > 128 ? 0 : (side > 64 ? 1 : 2);
+}
+
+// ACA of jobs given by class (count[c] jobs of class c, in class order), the classes side by side
+template <bool HALF>
+hbi_status launch_aca(const EntryGeo &g, const AcaJob *d_jobs, AcaOut *d_outs, const int *count, int64_t slot, int sms,
+                      double eps) {
+    BuildStreams bs;
+    DevScratch tmp;
+    hbi_status st = HBI_OK;
+    int at = 0;
+    for (int c = 0; c < ACA_CLASSES; at += count[c], ++c) {
+        if (count[c] == 0) continue;
+        cudaStream_t s = nullptr;
+        if ((st = bs.get(c, &s))) return st;
+        const AcaJob *j = d_jobs + at;
+        AcaOut *o = d_outs + at;
+        if (c == 0) aca_kernel<HALF, 256><<<(unsigned)count[c], 256, 0, s>>>(g, j, o, eps);
+        else if (c == 1) aca_kernel<HALF, 128><<<(unsigned)count[c], 128, 0, s>>>(g, j, o, eps);
+        else if (c == 2) aca_kernel<HALF, 64><<<(unsigned)count[c], 64, 0, s>>>(g, j, o, eps);
+        else {
+            int occ = 1;
+            HBI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, aca_full_kernel<HALF, 64>, 64, 0));
+            const int grid = std::min(count[c], sms * std::max(1, occ));
+            double *scratch = nullptr;
+            if ((st = tmp.alloc(&scratch, (size_t)grid * slot * sizeof(double)))) return st;
+            aca_full_kernel<HALF, 64><<<(unsigned)grid, 64, 0, s>>>(g, j, o, count[c], eps, scratch, slot);
+        }
+        HBI_CUDA_TRY(cudaGetLastError());
+    }
+    return bs.wait();
+}
 }  // namespace
 
 hbi_status device_build_factors(hbi_handle *h, const Tree &T, std::vector<Block> &blocks, double eps,
                                 std::vector<void *> &owned) {
-    EntryGeo g{h->d_geom, h->d_verts, h->d_rake, h->nv, h->op, h->nin, h->nout, h->mu, h->nu};
+    EntryGeo g{h->d_geom, h->d_verts, h->d_rake, h->nv, h->op, h->nin, h->nout, h->mu, h->nu, nullptr};
     int *d_bad = nullptr;
+    DevScratch edges;   // the edges' constants, for this build
+    EdgeConst *d_edges = nullptr;
     hbi_status st = dev_alloc(&d_bad, 1, owned);
+    if (!st) st = edges.alloc(&d_edges, (size_t)h->n * h->nv * sizeof(EdgeConst));
     if (st) return st;
+    edge_const_kernel<<<(unsigned)((h->n * h->nv + 127) / 128), 128>>>(g, h->n, d_edges);
+    HBI_CUDA_TRY(cudaGetLastError());
+    g.edges = reinterpret_cast<const double *>(d_edges);
     HBI_CUDA_TRY(cudaMemset(d_bad, 0, sizeof(int)));
 
     // ---- low-rank candidates: ACA with growing rank budgets
+    int dev = 0, sms = 1;
+    HBI_CUDA_TRY(cudaGetDevice(&dev));
+    HBI_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    std::vector<char> stepwise(blocks.size(), 0);   // not to be evaluated whole (a pair of it is singular)
     std::vector<int> pending;
     for (int b = 0; b < (int)blocks.size(); ++b)
         if (blocks[b].lowrank) pending.push_back(b);
@@ -279,6 +377,26 @@ hbi_status device_build_factors(hbi_handle *h, const Tree &T, std::vector<Block>
                 bytes += need;
                 ++pos;
             }
+            // by launch class, the largest blocks of a class first
+            auto cls = [&](int q) { return aca_class(jobs[q].tau_size, jobs[q].sig_size, stepwise[ids[q]]); };
+            std::vector<int> order(jobs.size());
+            for (size_t q = 0; q < order.size(); ++q) order[q] = (int)q;
+            std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+                const int cx = cls(x), cy = cls(y);
+                return cx < cy || (cx == cy && jobs[x].m + jobs[x].nc > jobs[y].m + jobs[y].nc);
+            });
+            std::vector<AcaJob> sorted;
+            std::vector<int> sorted_ids;
+            int count[ACA_CLASSES] = {};
+            int64_t slot = 0;
+            for (int q : order) {
+                sorted.push_back(jobs[q]);
+                sorted_ids.push_back(ids[q]);
+                ++count[cls(q)];
+                if (cls(q) == 3) slot = std::max<int64_t>(slot, (int64_t)jobs[q].m * jobs[q].nc);
+            }
+            jobs.swap(sorted);
+            ids.swap(sorted_ids);
             // one allocation for the batch's factors (kept until packing), one for flags
             size_t nd = 0, nf = 0;
             for (auto &J : jobs) { nd += (size_t)(J.m + J.nc) * J.rmax; nf += (size_t)(J.m + J.nc); }
@@ -300,11 +418,9 @@ hbi_status device_build_factors(hbi_handle *h, const Tree &T, std::vector<Block>
                 (st = tmp.alloc(&d_outs, jobs.size() * sizeof(AcaOut))))
                 return st;
             HBI_CUDA_TRY(cudaMemcpy(d_jobs, jobs.data(), jobs.size() * sizeof(AcaJob), cudaMemcpyHostToDevice));
-            if (h->half_space)
-                aca_kernel<true><<<(unsigned)jobs.size(), ACA_THREADS>>>(g, d_jobs, d_outs, eps);
-            else
-                aca_kernel<false><<<(unsigned)jobs.size(), ACA_THREADS>>>(g, d_jobs, d_outs, eps);
-            HBI_CUDA_TRY(cudaGetLastError());
+            if ((st = h->half_space ? launch_aca<true>(g, d_jobs, d_outs, count, slot, sms, eps)
+                                    : launch_aca<false>(g, d_jobs, d_outs, count, slot, sms, eps)))
+                return st;
             std::vector<AcaOut> outs(jobs.size());
             HBI_CUDA_TRY(cudaMemcpy(outs.data(), d_outs, outs.size() * sizeof(AcaOut), cudaMemcpyDeviceToHost));
             for (size_t q = 0; q < jobs.size(); ++q) {
@@ -317,7 +433,10 @@ hbi_status device_build_factors(hbi_handle *h, const Tree &T, std::vector<Block>
                     set_error("ACA did not converge within rank 2048 (injected)");
                     return HBI_ERR_ACA_FAIL;
                 }
-                if (outs[q].status == 0) {
+                if (outs[q].status == 4) {
+                    stepwise[ids[q]] = 1;
+                    pending.push_back(ids[q]);   // again in this pass
+                } else if (outs[q].status == 0) {
                     B.rank = outs[q].rank;
                     B.d_src = jobs[q].U;       // U column-major, leading dimension m
                     B.d_src2 = jobs[q].V;      // V column-major, leading dimension nc

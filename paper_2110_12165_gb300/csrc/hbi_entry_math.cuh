@@ -31,6 +31,13 @@ struct EntryGeo {
     const double *rake;   // permuted rake angle (single-component operators)
     int nv, op, nin, nout;
     double mu, nu;
+    const double *edges;  // permuted: EdgeConst of each element's nv edges (null: formed as needed)
+};
+
+// An edge's unit vector and length, formed once per element: an entry needs an edge's in four
+// loads instead of a square root and three divisions.
+struct EdgeConst {
+    double t[3], L;
 };
 
 __host__ __device__ __forceinline__ double dot3(const double *a, const double *b) {
@@ -52,13 +59,24 @@ __host__ __device__ __forceinline__ double tail_k2(double u, double r) {
     return (r * r + r * u + u * u) / (3.0 * r * r * r * (r + u));
 }
 
+__host__ __device__ __forceinline__ EdgeConst edge_const(const double *A, const double *B) {
+    EdgeConst e;
+    const double t[3] = {B[0] - A[0], B[1] - A[1], B[2] - A[2]};
+    e.L = sqrt(dot3(t, t));
+    for (int k = 0; k < 3; ++k) e.t[k] = t[k] / e.L;
+    return e;
+}
+
 // Adds one edge's contribution to beta for the two Burgers vectors b[0], b[1].
-// Returns false if the receiver lies on the edge itself.
-__host__ __device__ bool edge_beta(const double *x, const double *A, const double *B, const double (*b)[3],
-                          double nu, double (*beta)[9]) {
-    double t[3] = {B[0] - A[0], B[1] - A[1], B[2] - A[2]};
-    const double L = sqrt(dot3(t, t));
-    t[0] /= L; t[1] /= L; t[2] /= L;
+// Returns false if the receiver lies on the edge itself.  FP64 divisions and square roots are most
+// of its cost: each quotient is formed once, and the two cases of a receiver beyond one end of
+// the edge, which lanes of a warp meet side by side, take the same instructions (u1 is the nearer
+// end's distance along the edge, both counted away from the receiver).
+__host__ __device__ __forceinline__ bool edge_beta(const double *x, const double *A, const double *B,
+                                                   const double (*b)[3], const EdgeConst &ec, double nu,
+                                                   double (*beta)[9]) {
+    const double t[3] = {ec.t[0], ec.t[1], ec.t[2]};
+    const double L = ec.L;
     const double R0[3] = {x[0] - A[0], x[1] - A[1], x[2] - A[2]};
     const double RB[3] = {x[0] - B[0], x[1] - B[1], x[2] - B[2]};
     const double s0 = dot3(R0, t);
@@ -68,14 +86,12 @@ __host__ __device__ bool edge_beta(const double *x, const double *A, const doubl
     const double rA = sqrt(dot3(R0, R0)), rB = sqrt(dot3(RB, RB));
     double J0, K0, K2;
     bool ok = true;
-    if (uB >= 0.0) {
-        J0 = tail_j0(uB, rB) - tail_j0(uA, rA);
-        K0 = tail_k0(uB, rB) - tail_k0(uA, rA);
-        K2 = tail_k2(uB, rB) - tail_k2(uA, rA);
-    } else if (uA <= 0.0) {
-        J0 = tail_j0(-uA, rA) - tail_j0(-uB, rB);
-        K0 = tail_k0(-uA, rA) - tail_k0(-uB, rB);
-        K2 = tail_k2(-uA, rA) - tail_k2(-uB, rB);
+    const bool past = uB >= 0.0;
+    if (past || uA <= 0.0) {
+        const double u1 = past ? uB : -uA, r1 = past ? rB : rA, u2 = past ? uA : -uB, r2 = past ? rA : rB;
+        J0 = tail_j0(u1, r1) - tail_j0(u2, r2);
+        K0 = tail_k0(u1, r1) - tail_k0(u2, r2);
+        K2 = tail_k2(u1, r1) - tail_k2(u2, r2);
     } else {
         // receiver projects inside the edge: antiderivatives are odd, no cancellation
         if (!(d2 > 1e-20 * L * L)) ok = false;
@@ -86,9 +102,10 @@ __host__ __device__ bool edge_beta(const double *x, const double *A, const doubl
         K2 = uA * uA * uA / (3.0 * d2 * rA3) - uB * uB * uB / (3.0 * d2 * rB3);
     }
     const double rA3 = rA * rA * rA, rB3 = rB * rB * rB;
-    const double J1 = 1.0 / rB - 1.0 / rA;
+    const double iA = 1.0 / rA, iB = 1.0 / rB;
+    const double J1 = iB - iA;
     const double K1 = (1.0 / rB3 - 1.0 / rA3) / 3.0;
-    const double K3 = (-1.0 / rA + d2 / (3.0 * rA3)) - (-1.0 / rB + d2 / (3.0 * rB3));
+    const double K3 = (-iA + d2 / (3.0 * rA3)) - (-iB + d2 / (3.0 * rB3));
     const double I1[3] = {dv[0] * J0 + t[0] * J1, dv[1] * J0 + t[1] * J1, dv[2] * J0 + t[2] * J1};
     const double Cmu = 1.0 / (16.0 * M_PI * (1.0 - nu));
 #pragma unroll
@@ -300,7 +317,7 @@ __host__ __device__ void hs_correction(const EntryGeo &g, const double *x, int j
 // change (compression positive); columns = unit slip along source strike, source dip.
 // HALF: in the half space (full-space part + the correction above).
 template <bool HALF>
-__host__ __device__ bool pair_full(const EntryGeo &g, int i, int j, double T[3][2]) {
+__host__ __device__ __forceinline__ bool pair_full(const EntryGeo &g, int i, int j, double T[3][2]) {
     const double *gi = g.geom + 12 * (size_t)i, *gj = g.geom + 12 * (size_t)j;
     const double b[2][3] = {{gj[6], gj[7], gj[8]}, {gj[9], gj[10], gj[11]}};
     double beta[2][9];
@@ -308,9 +325,12 @@ __host__ __device__ bool pair_full(const EntryGeo &g, int i, int j, double T[3][
     for (int k = 0; k < 9; ++k) { beta[0][k] = 0.0; beta[1][k] = 0.0; }
     const double *vj = g.verts + (size_t)j * g.nv * 3;
     bool ok = true;
+#pragma unroll 1
     for (int a = 0; a < g.nv; ++a) {
         int a1 = (a + 1 == g.nv) ? 0 : a + 1;
-        ok &= edge_beta(gi, vj + 3 * a, vj + 3 * a1, b, g.nu, beta);
+        const EdgeConst ec = g.edges ? reinterpret_cast<const EdgeConst *>(g.edges)[(size_t)j * g.nv + a]
+                                     : edge_const(vj + 3 * a, vj + 3 * a1);
+        ok &= edge_beta(gi, vj + 3 * a, vj + 3 * a1, b, ec, g.nu, beta);
     }
     if (HALF) hs_correction(g, gi, j, b, beta);
     const double lam = 2.0 * g.mu * g.nu / (1.0 - 2.0 * g.nu);
@@ -339,7 +359,7 @@ __host__ __device__ bool pair_full(const EntryGeo &g, int i, int j, double T[3][
 
 // Operator entries E[c_out][c_in] (n_out x n_in of the operator form).
 template <bool HALF>
-__host__ __device__ bool pair_op(const EntryGeo &g, int i, int j, double E[3][2]) {
+__host__ __device__ __forceinline__ bool pair_op(const EntryGeo &g, int i, int j, double E[3][2]) {
     double T[3][2];
     bool ok = pair_full<HALF>(g, i, j, T);
     if (g.op == HBI_OP_VEC_FULL || g.op == HBI_OP_VEC_SHEAR) {

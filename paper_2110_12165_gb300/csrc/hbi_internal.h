@@ -65,6 +65,34 @@ struct DevScratch {
     }
 };
 
+// Streams of one build step, for launches that run side by side.  They start after the work the
+// legacy default stream holds, wait() returns when all of them are done, and they go with the
+// holder (every return path; their work is waited for first).
+struct BuildStreams {
+    static constexpr int MAX = 8;
+    cudaStream_t s[MAX] = {};
+    hbi_status get(int i, cudaStream_t *out) {
+        if (!s[i]) HBI_CUDA_TRY(cudaStreamCreate(&s[i]));   // ordered with the legacy default stream
+        *out = s[i];
+        return HBI_OK;
+    }
+    hbi_status wait() {
+        for (cudaStream_t q : s)
+            if (q) HBI_CUDA_TRY(cudaStreamSynchronize(q));
+        return HBI_OK;
+    }
+    BuildStreams() = default;
+    BuildStreams(const BuildStreams &) = delete;
+    BuildStreams &operator=(const BuildStreams &) = delete;
+    ~BuildStreams() {
+        for (cudaStream_t q : s)
+            if (q) {
+                cudaStreamSynchronize(q);
+                cudaStreamDestroy(q);
+            }
+    }
+};
+
 // ------------------------------------------------------------ dependent launches
 // The kernels of a product (and of an attempt) are launched with programmatic stream
 // serialisation: a kernel may start once every CTA of the one before it has exited, before that

@@ -19,10 +19,15 @@
 
 namespace hbi {
 
-constexpr int RC_THREADS = 256;
 constexpr int RC_RMAX = 48;          // blocks of higher rank are left as they are
 constexpr int RC_TILE = 32;          // rows per tile of the Gram and update passes
-constexpr int RC_PAIRS = (RC_RMAX * (RC_RMAX + 1) / 2 + RC_THREADS - 1) / RC_THREADS;
+
+// A block's work is a chain of short passes with barriers between them, so an SM needs several
+// CTAs to hide them.  What it can hold is set by the rank (six r x r matrices in shared memory), so
+// the blocks are launched in classes of their rank, each sized for its largest (threads per CTA
+// and CTAs per SM), the large blocks of a class first.  With one class for all, 256 threads of 254
+// registers, one CTA an SM: 127 ms for the 9,086 blocks of a 20,022-element fault; with the
+// classes and eight lanes a Jacobi pair 64 ms.  The results do not depend on the class.
 
 struct RecompJob {
     double *U, *V;       // column-major, leading dimensions m and n, rank r (updated in place)
@@ -30,7 +35,9 @@ struct RecompJob {
 };
 
 // G = X^T X for X (len x r, column-major); tile = RC_TILE x r scratch in shared memory.
+template <int RMAX, int THREADS>
 __device__ void gram(const double *X, int len, int r, double *G, double *tile) {
+    constexpr int RC_PAIRS = (RMAX * (RMAX + 1) / 2 + THREADS - 1) / THREADS;
     const int npair = r * (r + 1) / 2;
     int pa[RC_PAIRS], pb[RC_PAIRS];
     double acc[RC_PAIRS];
@@ -106,20 +113,21 @@ __device__ bool chol_scaled(double *G, int r, double *d, int *s_ok) {
 }
 
 // shared memory (doubles): RU, RV, C, Z, TU, TV (r*r each), tile (RC_TILE*r), sv (r)
-__global__ void __launch_bounds__(RC_THREADS) recompress_kernel(const RecompJob *jobs, int *new_rank, double tol) {
+template <int RMAX, int THREADS, int PER_SM>
+__global__ void __launch_bounds__(THREADS, PER_SM) recompress_kernel(const RecompJob *jobs, int *new_rank, double tol) {
     extern __shared__ __align__(16) double sm[];
     __shared__ int s_ok, s_keep;
-    __shared__ int s_order[RC_RMAX];
-    __shared__ double s_d[RC_RMAX];
+    __shared__ int s_order[RMAX];
+    __shared__ double s_d[RMAX];
     const RecompJob J = jobs[blockIdx.x];
     const int r = J.r, rr = r * r;
     double *RU = sm, *RV = RU + rr, *C = RV + rr, *Z = C + rr, *TU = Z + rr, *TV = TU + rr;
     double *tile = TV + rr, *sv = tile + RC_TILE * r;
     if (threadIdx.x == 0) new_rank[blockIdx.x] = r;
-    if (r < 2 || r > RC_RMAX) return;
-    gram(J.U, J.m, r, RU, tile);
+    if (r < 2 || r > RMAX) return;
+    gram<RMAX, THREADS>(J.U, J.m, r, RU, tile);
     if (!chol_scaled(RU, r, s_d, &s_ok)) return;
-    gram(J.V, J.n, r, RV, tile);
+    gram<RMAX, THREADS>(J.V, J.n, r, RV, tile);
     if (!chol_scaled(RV, r, s_d, &s_ok)) return;
     // core C = R_U R_V^T (column-major: C[i + j r]), Z = I
     for (int e = threadIdx.x; e < rr; e += blockDim.x) {
@@ -130,43 +138,63 @@ __global__ void __launch_bounds__(RC_THREADS) recompress_kernel(const RecompJob 
         Z[e] = (i == j) ? 1.0 : 0.0;
     }
     __syncthreads();
-    // one-sided Jacobi on the columns of C; disjoint pairs of one round-robin round per step
+    // one-sided Jacobi on the columns of C; the disjoint pairs of one round-robin round per step,
+    // eight lanes a pair.  A pair's angle (square roots and divisions, about 100 FP64 instructions)
+    // costs as much as its dot products and rotations together, and a warp instruction costs the
+    // same for one pair as for four.  Lane s of a pair holds rows s, s + 8, s + 16 and s + 24, so
+    // that the sums add up as over 32 lanes of a row each.
     const int np = (r + 1) & ~1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int grp = lane >> 3, s8 = lane & 7;
     for (int sweep = 0; sweep < 30; ++sweep) {
         if (threadIdx.x == 0) s_ok = 0;   // "a rotation happened in this sweep"
         __syncthreads();
         for (int round = 0; round < np - 1; ++round) {
-            for (int k = warp; k < np / 2; k += nw) {
+            for (int k0 = 4 * warp; k0 < np / 2; k0 += 4 * nw) {
+                const int k = k0 + grp;
                 int p = k == 0 ? 0 : (k - 1 + round) % (np - 1) + 1;
                 const int kk = np - 1 - k;
                 int q = kk == 0 ? 0 : (kk - 1 + round) % (np - 1) + 1;
                 if (p > q) { const int t = p; p = q; q = t; }
-                if (q >= r) continue;
-                double a = 0.0, b = 0.0, c = 0.0;
-                for (int i = lane; i < r; i += 32) {
-                    const double x = C[i + p * r], y = C[i + q * r];
-                    a += x * x; b += y * y; c += x * y;
-                }
+                const bool on = k < np / 2 && q < r;
+                double *Cp = C + (on ? p : 0) * r, *Cq = C + (on ? q : 0) * r;
+                double a4[4], b4[4], c4[4];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
+                for (int e = 0; e < 4; ++e) {
+                    const int i = s8 + 8 * e;
+                    double a = 0.0, b = 0.0, c = 0.0;
+                    for (int w = i; w < r; w += 32) {
+                        const double x = Cp[w], y = Cq[w];
+                        a += x * x; b += y * y; c += x * y;
+                    }
+                    a4[e] = a; b4[e] = b; c4[e] = c;
+                }
+                double a = (a4[0] + a4[2]) + (a4[1] + a4[3]);
+                double b = (b4[0] + b4[2]) + (b4[1] + b4[3]);
+                double c = (c4[0] + c4[2]) + (c4[1] + c4[3]);
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) {
                     a += __shfl_xor_sync(0xffffffffu, a, o);
                     b += __shfl_xor_sync(0xffffffffu, b, o);
                     c += __shfl_xor_sync(0xffffffffu, c, o);
                 }
-                if (c == 0.0 || fabs(c) <= 1e-15 * sqrt(a * b)) continue;
+                const bool rot = on && !(c == 0.0 || fabs(c) <= 1e-15 * sqrt(a * b));
+                if (!__any_sync(0xffffffffu, rot)) continue;
                 const double zeta = (b - a) / (2.0 * c);
                 const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
                 const double cs = 1.0 / sqrt(1.0 + t * t), sn = cs * t;
-                for (int i = lane; i < r; i += 32) {
-                    const double x = C[i + p * r], y = C[i + q * r];
-                    C[i + p * r] = cs * x - sn * y;
-                    C[i + q * r] = sn * x + cs * y;
-                    const double u = Z[i + p * r], v = Z[i + q * r];
-                    Z[i + p * r] = cs * u - sn * v;
-                    Z[i + q * r] = sn * u + cs * v;
+                if (rot) {
+                    double *Zp = Z + p * r, *Zq = Z + q * r;
+                    for (int i = s8; i < r; i += 8) {
+                        const double x = Cp[i], y = Cq[i];
+                        Cp[i] = cs * x - sn * y;
+                        Cq[i] = sn * x + cs * y;
+                        const double u = Zp[i], v = Zq[i];
+                        Zp[i] = cs * u - sn * v;
+                        Zq[i] = sn * u + cs * v;
+                    }
+                    if (s8 == 0) s_ok = 1;
                 }
-                if (lane == 0) s_ok = 1;
             }
             __syncthreads();
         }
@@ -243,30 +271,66 @@ __global__ void __launch_bounds__(RC_THREADS) recompress_kernel(const RecompJob 
     if (threadIdx.x == 0) new_rank[blockIdx.x] = rk;
 }
 
+namespace {
+template <int RMAX, int THREADS, int PER_SM>
+hbi_status recompress_class(const RecompJob *d_jobs, int *d_rank, int njobs, double tol, cudaStream_t s) {
+    if (njobs == 0) return HBI_OK;
+    const int smem = (6 * RMAX * RMAX + RC_TILE * RMAX + RMAX) * (int)sizeof(double);
+    auto *k = recompress_kernel<RMAX, THREADS, PER_SM>;
+    HBI_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    k<<<(unsigned)njobs, THREADS, smem, s>>>(d_jobs, d_rank, tol);
+    HBI_CUDA_TRY(cudaGetLastError());
+    return HBI_OK;
+}
+}  // namespace
+
 // Recompress every low-rank block of rank 2..RC_RMAX; updates ranks in place (the first
 // r' columns of the same U and V storage hold the new factors).
 hbi_status recompress_lowrank(std::vector<Block> &blocks, double tol) {
     std::vector<RecompJob> jobs;
     std::vector<int> ids;
-    int rmax = 0;
     for (size_t b = 0; b < blocks.size(); ++b) {
-        Block &B = blocks[b];
-        if (!B.lowrank || B.rank < 2 || B.rank > RC_RMAX) continue;
+        const Block &B = blocks[b];
+        if (B.lowrank && B.rank >= 2 && B.rank <= RC_RMAX) ids.push_back((int)b);
+    }
+    if (ids.empty()) return HBI_OK;
+    // classes of rank, the highest first; by decreasing size inside a class
+    auto cls = [&](int b) { return (RC_RMAX - blocks[b].rank) / 8; };   // 41-48, 33-40, 25-32, 17-24, 9-16, 2-8
+    std::stable_sort(ids.begin(), ids.end(), [&](int x, int y) {
+        const int cx = cls(x), cy = cls(y);
+        return cx < cy || (cx == cy && blocks[x].m + blocks[x].nc > blocks[y].m + blocks[y].nc);
+    });
+    int count[6] = {0, 0, 0, 0, 0, 0};
+    for (int b : ids) {
+        const Block &B = blocks[b];
         jobs.push_back(RecompJob{const_cast<double *>(B.d_src), const_cast<double *>(B.d_src2), (int)B.m, (int)B.nc,
                                  B.rank});
-        ids.push_back((int)b);
-        rmax = std::max(rmax, B.rank);
+        ++count[cls(b)];
     }
-    if (jobs.empty()) return HBI_OK;
-    const size_t smem = ((size_t)6 * rmax * rmax + (size_t)RC_TILE * rmax + rmax) * sizeof(double);
-    HBI_CUDA_TRY(cudaFuncSetAttribute(recompress_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     RecompJob *d_jobs = nullptr;
     int *d_rank = nullptr;
     DevScratch tmp;
     hbi_status st;
     if ((st = tmp.upload(&d_jobs, jobs)) || (st = tmp.alloc(&d_rank, jobs.size() * sizeof(int)))) return st;
-    recompress_kernel<<<(unsigned)jobs.size(), RC_THREADS, smem>>>(d_jobs, d_rank, tol);
-    HBI_CUDA_TRY(cudaGetLastError());
+    BuildStreams bs;   // the classes side by side, so that one's last blocks do not leave SMs idle
+    int at = 0;
+    for (int c = 0; c < 6 && !st; at += count[c], ++c) {
+        const RecompJob *j = d_jobs + at;
+        int *r = d_rank + at;
+        cudaStream_t s = nullptr;
+        if (count[c] == 0) continue;
+        if ((st = bs.get(c, &s))) break;
+        switch (c) {
+            case 0: st = recompress_class<48, 192, 1>(j, r, count[c], tol, s); break;
+            case 1: st = recompress_class<40, 160, 2>(j, r, count[c], tol, s); break;
+            case 2: st = recompress_class<32, 128, 3>(j, r, count[c], tol, s); break;
+            case 3: st = recompress_class<24, 96, 6>(j, r, count[c], tol, s); break;
+            case 4: st = recompress_class<16, 64, 12>(j, r, count[c], tol, s); break;
+            default: st = recompress_class<8, 32, 16>(j, r, count[c], tol, s); break;
+        }
+    }
+    const hbi_status st2 = bs.wait();
+    if (st || st2) return st ? st : st2;
     std::vector<int> nr(jobs.size());
     HBI_CUDA_TRY(cudaMemcpy(nr.data(), d_rank, nr.size() * sizeof(int), cudaMemcpyDeviceToHost));
     for (size_t q = 0; q < jobs.size(); ++q) {
