@@ -259,7 +259,7 @@ hbi_status hbi_matvec_noalloc(hbi_handle *h, const double *d_x, double *d_y, hbi
  * conditions, or the stages of several runs).
  * d_X: k x n_in N doubles, right-hand side r at d_X[r n_in N + c N + i] (each one laid out
  * as the d_x of hbi_matvec); d_Y: k x n_out N doubles, the same way.  1 <= k <= 64 (k is
- * padded to a multiple of 16 internally).  Work buffers for k are allocated on the first
+ * padded to 16, 32 or 64 internally).  Work buffers for k are allocated on the first
  * call with that size and kept by the handle.  Synchronises the stream.
  * Errors: INVALID_ARG (NULL pointers, k out of range, handle without the panels), CUDA,
  * TIMEOUT.
@@ -270,7 +270,8 @@ hbi_status hbi_matvec_multi(hbi_handle *h, int k, const double *d_X, double *d_Y
  * hbi_time_multi -- device time of the multi-RHS product on the input of the handle's last
  * hbi_matvec_multi call with the same k (call that first), averaged over n_rep back-to-back
  * products with CUDA events recorded on `stream`: out3[0] = V^T phase, out3[1] = U t + dense
- * phase, out3[2] = both (ms; the input and output permutations are not included).
+ * phase, out3[2] = both (ms; the splits of the inputs are included, the input and output
+ * permutations are not).
  * Errors: INVALID_ARG, CUDA, TIMEOUT.
  */
 hbi_status hbi_time_multi(hbi_handle *h, int k, int n_rep, double *out3, hbi_stream stream);

@@ -13,16 +13,18 @@
 // FP32 near field of HBI_MIXED as an FP16 pair hi + 2^-11 lo), packed at build time in the
 // canonical no-swizzle K-major tcgen05 layout (8 x 8 core matrices of 128 contiguous bytes),
 // in chunks of MR_CW columns, so that one cp.async.bulk lands a chunk in shared memory ready
-// for the MMA.  B = the inputs, FP32 in HBM, scaled per right-hand side to FP16 range and
-// split into hi + 2^-11 lo FP16 parts (22 significant bits) in the canonical MN-major layout.
-// The MMA (kind::f16, M = 128 panel rows, N = k padded to 16, K = 16) accumulates in FP32 in
-// tensor memory: D1 = A_hi B_hi and D2 = A_hi B_lo + A_lo B_hi; y = (D1 + 2^-11 D2) / s.
+// for the MMA.  B = the input rows, scaled per right-hand side to FP16 range and split into
+// hi + 2^-11 lo FP16 parts (22 significant bits) once per row (mr_split_kernel), [hi | lo] of one
+// row side by side; a chunk's rows are fetched by index with 16-byte asynchronous copies straight
+// into the swizzled MN-major layout the MMA reads.  The MMA (kind::f16, M = 128 panel rows,
+// K = 16) accumulates in FP32 in tensor memory: D1 = A_hi B_hi and D2 = A_hi B_lo + A_lo B_hi;
+// y = (D1 + 2^-11 D2) / s.
 //
-// Persistent CTAs, warp-specialised: a producer warp streams the A pieces into a ring of MR_SA
-// shared-memory stages (bulk copies on mbarriers), four warps convert one B chunk each into
-// a ring of MR_SB stages, four warps run the epilogue (tcgen05.ld, one TMEM lane per panel
-// row) from one of two accumulators while the next task's MMAs fill the other, and one warp
-// allocates tensor memory and issues the MMAs, releasing each stage with tcgen05.commit.
+// Persistent CTAs, warp-specialised: one thread streams the A pieces into a ring of
+// shared-memory stages (bulk copies on mbarriers), four warps gather the B chunks into a second
+// ring, one warp allocates tensor memory and issues the MMAs, releasing each stage with
+// tcgen05.commit, and four warps run the epilogue (tcgen05.ld, one TMEM lane per panel row)
+// from one of two accumulators while the next task's MMAs fill the other.
 // Every wait is bounded; a CTA that gives up raises the error flag, lets its copies and MMAs
 // in flight finish and frees its tensor memory.
 #include <cuda_fp16.h>
@@ -31,36 +33,28 @@
 #include <algorithm>
 #include <cstring>
 #include <map>
+#include <type_traits>
 #include <vector>
 
 #include "hbi_internal.h"
 
 namespace hbi {
 
-#ifndef HBI_MR_CW
-#define HBI_MR_CW 64
-#endif
-
-#ifndef HBI_MR_SB
-#define HBI_MR_SB 4
-#endif
-constexpr int MR_CW = HBI_MR_CW;                   // K columns per chunk
-// A ring stages (one panel piece of 16 KB each): three for 32 right-hand sides, so that two CTAs
-// share an SM (measured 1.9x faster than one CTA with four), four otherwise
-__host__ __device__ constexpr int mr_stages_a(int kp) { return kp == 32 ? 3 : 4; }
-constexpr int MR_SB = HBI_MR_SB;                   // B ring stages
-constexpr int MR_GW = 4;                           // converter warps (and epilogue warps: TMEM lanes 0..127)
-constexpr int MR_SS = MR_SB;                       // staging stages (one per B stage)
-// Converter warp w takes the chunks g = w (mod MR_GW); a stage must come back to the same warp
-// (MR_SB, MR_SS multiples of MR_GW), so that no warp waits on a stage whose previous phase
-// another warp has not yet consumed (a parity wait cannot tell two phases apart).
-static_assert(MR_SB % MR_GW == 0 && MR_SS % MR_GW == 0, "B and staging stages: multiples of the converter warps");
+constexpr int MR_CW = 64;                          // K columns per chunk
+// Ring stages of A (a panel piece of 16 KB each) and of B (MR_CW rows of 4 kp bytes): what lets two
+// CTAs share an SM, so that one's epilogue and waits run beside the other's MMAs (64 right-hand
+// sides at 40,000 elements, both phases: 316 us; one CTA with seven and six stages 420 us, two
+// with three and three 346 us; 32 right-hand sides 260 us, three CTAs 294 us, one 363 us).
+__host__ __device__ constexpr int mr_stages_a(int kp) { return kp == 64 ? 4 : 5; }
+__host__ __device__ constexpr int mr_stages_b(int kp) { return kp == 16 ? 6 : 3; }
+constexpr int MR_GW = 4;                           // epilogue warps (TMEM lanes 0..127)
+constexpr int MR_BW = 4;                           // B producer warps
 static_assert(mr_stages_a(16) >= 2 && mr_stages_a(32) >= 2 && mr_stages_a(64) >= 2,
               "a dense chunk with a lo part holds two A stages");
-constexpr int MR_THREADS = 32 * (2 * MR_GW + 3);   // converter, epilogue, A producer, MMA and B producer warps
+constexpr int MR_THREADS = 32 * (MR_GW + 2 + MR_BW);   // epilogue, A producer, MMA and B producer warps
 constexpr int MR_ROWS = 128;                       // MMA M: panel rows of a task
 constexpr int MR_A_STAGE = MR_ROWS * MR_CW * 2;    // bytes: one part (hi or lo) of a 128-row chunk
-constexpr int MR_KP_MAX = 64;                      // right-hand sides per call (padded to 16)
+constexpr int MR_KP_MAX = 64;                      // right-hand sides per call (padded to 16, 32 or 64)
 constexpr int MR_KSLICE = 2048;                    // V^T: widest K of one task (wider groups are cut)
 constexpr unsigned long long MR_WAIT_NS = 1000000000ull;   // 1 s
 
@@ -69,7 +63,7 @@ constexpr unsigned long long MR_WAIT_NS = 1000000000ull;   // 1 s
 // kl factor columns (U or V^T), each segment a multiple of 16 and cut into chunks of MR_CW.
 struct MrTask {
     int64_t a_off;     // byte offset of the first chunk in the panel stream
-    int64_t g_off;     // UY: offset of the unit's gather list; V^T: first X row of the group
+    int64_t g_off;     // offset of the task's B row indices (MR_CW per chunk)
     int64_t out_off;   // first output row (V^T: row of T inside xt; UY: row of yp)
     int64_t s_off;     // V^T: rowscale index of row 0; UY: -1
     int rows;          // 1..128
@@ -77,8 +71,6 @@ struct MrTask {
     int kreal;         // V^T: the group's columns (the padding gathers zeros)
     int lo;            // the dense chunks carry a lo part
     int partial;       // V^T: a K slice of a wide column group; its rows are partial sums
-    int nd_real;       // dense columns before the padding of the dense segment (V^T: 0)
-    int nl_real;       // factor columns before the padding of the factor segment (V^T: kreal)
 };
 
 // A V^T row tile of a wide column group, cut into nsl K slices: slice q wrote its partial rows
@@ -86,13 +78,6 @@ struct MrTask {
 struct MrSplit {
     int64_t t_row, p_row;
     int rows, nsl;
-};
-
-// One run of the B gather: len consecutive xt rows from row src land in the chunk's staging
-// buffer at columns [dst, dst + len) (one bulk copy of len x KP FP32 words).
-struct MrRun {
-    int64_t src;
-    int len, dst;
 };
 
 }  // namespace hbi
@@ -106,15 +91,7 @@ struct hbi::MultiRhs {
     MrSplit *d_split = nullptr;   // V^T row tiles cut along K (reduced after the V^T phase)
     int n_split = 0;
     int64_t n_prow = 0;           // partial rows after T in xt
-    // B gather runs of every chunk, per phase: host copies in task order (first run of each
-    // task's chunk c at h_crun[p][c_first[task] + c]), and on the device in the order in which
-    // the CTAs of a grid of `layout_grid` take the chunks (d_crun[p][d_cta[p][b] + g] is the
-    // first run of chunk g of CTA b)
-    std::vector<MrRun> h_runs[2];
-    std::vector<int64_t> h_crun[2], h_cfirst[2];
-    MrRun *d_runs[2] = {nullptr, nullptr};
-    int64_t *d_crun[2] = {nullptr, nullptr}, *d_cta[2] = {nullptr, nullptr};
-    int layout_grid = 0;
+    int *d_bidx = nullptr;        // B row indices of every task's chunks (rows of x16; padding: its zero row)
     float *d_cscale = nullptr;    // per X row: the scale of its dense columns (largest over the blocks)
     int *d_iperm = nullptr;       // original element -> permuted position
     float *d_rowscale = nullptr;  // V^T output row scales (sv su)
@@ -125,9 +102,12 @@ struct hbi::MultiRhs {
     // per-call buffers, sized for kp_cap right-hand sides
     int kp_cap = 0;
     float *d_xt = nullptr, *d_yp = nullptr;
+    __half *d_x16 = nullptr;      // rows of X, of X with the dense column scales and of T, each [hi | lo], and a row of zeros
+    int row_kp = 0;               // the row length the grid and the row of zeros are for
+    int zeroed = 0;               // the row of zeros is written
     unsigned *d_vmax = nullptr;   // per right-hand side: [0, 64) max |x|, [64, 128) max |t|,
                                   // [128, 192) max |x| x its row's dense column scale
-    int *d_err = nullptr;
+    int *h_err = nullptr;         // error flag of bounded device waits (pinned; the kernels write it)
     int64_t bytes_panels_alg = 0;     // stored entries (hi + lo for the FP32 near field) + scales
     int64_t vec_bytes_per_rhs = 0;    // x read, t written and read, y written (FP32)
     double flops_per_rhs = 0;         // 2 x (dense + U + V entries)
@@ -191,11 +171,20 @@ __device__ __forceinline__ void mr_bulk(void *dst, const void *src, unsigned byt
                  "l"(src), "r"(bytes), "r"(mr_smem(b))
                  : "memory");
 }
-// Shared-memory matrix descriptor, no swizzle: start address, LBO = byte stride between core
-// matrices along K, SBO = byte stride between 8-row (M or N) groups; version 1 (bits 46-47).
-__device__ __forceinline__ uint64_t mr_desc(unsigned saddr, unsigned lbo, unsigned sbo) {
+__device__ __forceinline__ void mr_copy16(unsigned dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// arrives on the barrier once the thread's copies so far have landed
+__device__ __forceinline__ void mr_copy_arrive(uint64_t *b) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(mr_smem(b)) : "memory");
+}
+// Shared-memory matrix descriptor: start address, LBO and SBO byte strides, version 1 (bits
+// 46-47), swizzle mode (bits 61-63: 0 none, 2 128-byte, 4 64-byte).  No swizzle, K-major: LBO
+// between core matrices along K, SBO between 8-row groups.  Swizzled, MN-major: LBO between
+// atoms along N (one swizzle row of N elements each), SBO between groups of 8 K rows.
+__device__ __forceinline__ uint64_t mr_desc(unsigned saddr, unsigned lbo, unsigned sbo, unsigned swizzle) {
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
+           ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46) | ((uint64_t)swizzle << 61);
 }
 __device__ __forceinline__ void mr_mma(unsigned d_tmem, uint64_t a, uint64_t b, unsigned idesc, unsigned acc) {
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -261,56 +250,88 @@ __device__ __forceinline__ float mr_scale_for(float m) {
     return ldexpf(1.0f, 14 - c);
 }
 
+// The scale of right-hand side r: of the V^T phase from max |x|, of the UY phase from the larger of
+// max |x| with the dense column scales and max |t|.
+__device__ __forceinline__ float mr_phase_scale(const unsigned *vmax, int vt, int r) {
+    const float m = vt ? __uint_as_float(vmax[r]) : fmaxf(__uint_as_float(vmax[128 + r]), __uint_as_float(vmax[64 + r]));
+    return mr_scale_for(m);
+}
+
+// Rows [row0, row0 + nrows) of xt (KP FP32 words) times the phase's scales into x16 rows [hi | lo]:
+// hi = fp16(b), lo = fp16((b - hi) 2^11), b = x s.  Eight right-hand sides a thread.  One pass over
+// the inputs of a phase (bound by its traffic: 8 KP bytes a row) in place of a conversion of every
+// gathered row in the product kernel, where each row serves several chunks.
+template <int KP>
+__global__ void mr_split_kernel(const float *xt, const unsigned *vmax, int vt, int64_t row0, int64_t nrows,
+                                __half *x16) {
+    constexpr int PER = KP / 8;   // threads a row
+    pdl_wait();
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int r0 = 8 * (int)(t0 % PER);   // stride is a multiple of PER
+    float sc[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) sc[q] = mr_phase_scale(vmax, vt, r0 + q);
+    for (int64_t e = t0; e < nrows * PER; e += stride) {
+        const int64_t row = row0 + e / PER;
+        const float4 u = *reinterpret_cast<const float4 *>(xt + row * KP + r0);
+        const float4 v = *reinterpret_cast<const float4 *>(xt + row * KP + r0 + 4);
+        const float xs[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+        __align__(16) __half hi[8], lo[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float b = xs[q] * sc[q];
+            hi[q] = __float2half_rn(b);
+            lo[q] = __float2half_rn((b - __half2float(hi[q])) * 2048.0f);
+        }
+        *reinterpret_cast<uint4 *>(x16 + row * 2 * KP + r0) = *reinterpret_cast<const uint4 *>(hi);
+        *reinterpret_cast<uint4 *>(x16 + row * 2 * KP + KP + r0) = *reinterpret_cast<const uint4 *>(lo);
+    }
+}
+
 // ------------------------------------------------------------------ the product kernel
-// vt = 1: V^T phase (B = X rows g_off + col, outputs T rows scaled by rowscale, max |t| per
-// right-hand side into vmax[64 + r]); vt = 0: UY phase (B = gathered xt rows, outputs yp).
-// Warp 10 copies each chunk's B rows (FP32, runs of consecutive xt rows, one bulk copy per run)
-// into staging stage g (mod MR_SS) of the CTA's chunk sequence; converter warp g (mod 4) scales
-// and splits them into FP16 hi / lo B stage g (mod MR_SB); warps 4-7 run the epilogue from one
-// of two tensor-memory accumulators while the MMAs of the next task fill the other; warp 8
-// streams the A pieces; warp 9 allocates tensor memory and issues the MMAs.
+// vt = 1: V^T phase (outputs T rows scaled by rowscale, max |t| per right-hand side into
+// vmax[64 + r]); vt = 0: UY phase (outputs yp).  Warps 0-3 run the epilogue from one of two
+// tensor-memory accumulators while the MMAs of the next task fill the other; warp 4 streams the A
+// pieces (which depend on the operator alone, so it does not wait for the kernels before); warp
+// 5 allocates tensor memory and issues the MMAs; warps 6-9 gather each chunk's B rows by index.
 template <int KP>
 __global__ void __launch_bounds__(MR_THREADS, 1)
     mr_kernel(const MrTask *__restrict__ tasks, int ntasks, int vt, const unsigned char *__restrict__ panels,
-              const MrRun *__restrict__ runs, int64_t n_runs, const int64_t *__restrict__ crun,
-              const int64_t *__restrict__ cta, const float *__restrict__ rowscale, float *xt, float *out, unsigned *vmax,
-              int *err) {
-    constexpr int MR_SA = mr_stages_a(KP);     // A ring stages
-    constexpr int BSTAGE = MR_CW * KP * 2;    // bytes of one FP16 B part (hi or lo)
-    constexpr int SSTAGE = MR_CW * KP * 4;    // bytes of one FP32 staging stage
+              const __half *x16, const int *__restrict__ bidx, const float *__restrict__ rowscale,
+              float *out, unsigned *vmax, int *err) {
+    constexpr int MR_SA = mr_stages_a(KP), MR_SB = mr_stages_b(KP);   // ring stages
+    constexpr int ROWB = 4 * KP < 128 ? 4 * KP : 128;   // bytes of a K row in one swizzle atom
+    constexpr int NATOM = 4 * KP / ROWB;                // atoms along N: one, or hi and lo for KP = 64
+    constexpr int BATOM = MR_CW * ROWB;                 // bytes of an atom column of a chunk
+    constexpr int BSTAGE = NATOM * BATOM;
+    constexpr unsigned SWZ = ROWB == 128 ? 2u : 4u;
     constexpr unsigned TCOLS = 4 * KP <= 64 ? 64 : (4 * KP <= 128 ? 128 : 256);   // 2 accumulators x (D1 | D2)
     extern __shared__ __align__(1024) unsigned char mr_sm[];
     unsigned char *sA = mr_sm;                                        // MR_SA x MR_A_STAGE
-    unsigned char *sB = sA + MR_SA * MR_A_STAGE;                      // MR_SB x (hi | lo)
-    unsigned char *sS = sB + MR_SB * 2 * BSTAGE;                      // MR_SS x staging
-    __shared__ uint64_t a_full[MR_SA], a_empty[MR_SA], b_full[MR_SB], b_empty[MR_SB], s_full[MR_SS], s_empty[MR_SS];
+    unsigned char *sB = sA + MR_SA * MR_A_STAGE;                      // MR_SB x BSTAGE
+    __shared__ uint64_t a_full[MR_SA], a_empty[MR_SA], b_full[MR_SB], b_empty[MR_SB];
     __shared__ uint64_t acc_full[2], acc_empty[2], fin;
     __shared__ unsigned s_taddr;
-    __shared__ __align__(16) float s_scale[KP];
     __shared__ float s_inv[KP];
     __shared__ unsigned s_tmax[KP];
     __shared__ volatile int s_fail;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int W_EPI = MR_GW, W_PROD = 2 * MR_GW, W_MMA = 2 * MR_GW + 1, W_BPROD = 2 * MR_GW + 2;
+    constexpr int W_PROD = MR_GW, W_MMA = MR_GW + 1, W_BPROD = MR_GW + 2;
+    if (mr_smem(mr_sm) % 1024u != 0) {   // the swizzle goes by the address
+        if (threadIdx.x == 0) *(volatile int *)err = 1;
+        return;
+    }
 
     if (threadIdx.x == 0) {
         s_fail = 0;
         for (int s = 0; s < MR_SA; ++s) { mr_bar_init(&a_full[s], 1); mr_bar_init(&a_empty[s], 1); }
-        for (int s = 0; s < MR_SB; ++s) { mr_bar_init(&b_full[s], 32); mr_bar_init(&b_empty[s], 1); }
-        for (int s = 0; s < MR_SS; ++s) { mr_bar_init(&s_full[s], 1); mr_bar_init(&s_empty[s], 32); }
+        for (int s = 0; s < MR_SB; ++s) { mr_bar_init(&b_full[s], 32 * MR_BW); mr_bar_init(&b_empty[s], 1); }
         for (int s = 0; s < 2; ++s) { mr_bar_init(&acc_full[s], 1); mr_bar_init(&acc_empty[s], 32 * MR_GW); }
         mr_bar_init(&fin, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (threadIdx.x < KP) {
-        const int r = threadIdx.x;
-        const float xm = __uint_as_float(vmax[r]);
-        const float m = vt ? xm : fmaxf(__uint_as_float(vmax[128 + r]), __uint_as_float(vmax[64 + r]));
-        const float s = mr_scale_for(m);
-        s_scale[r] = s;
-        s_inv[r] = 1.0f / s;
-        s_tmax[r] = 0u;
-    }
+    if (threadIdx.x < KP) s_tmax[threadIdx.x] = 0u;
     if (warp == W_MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(mr_smem(&s_taddr)),
                      "r"(TCOLS)
@@ -355,62 +376,59 @@ __global__ void __launch_bounds__(MR_THREADS, 1)
                 }
             }
         }
-    } else if (warp == W_BPROD) {
-        // ---------------------------------------------------------------- B producer (whole warp)
-        // This CTA's chunks g = 0 .. nchk - 1 take the runs [crun[c0 + g], crun[c0 + g + 1]).  The
-        // lanes hold 32 chunk boundaries and three windows of 32 runs (a 64-column chunk has at
-        // most 64 runs, so it lies inside the three), with the next boundaries and the third
-        // window loaded ahead of use; each lane issues the bulk copies of the runs it holds.
-        const int64_t c0 = cta[blockIdx.x];
-        const int nchk = (int)(cta[blockIdx.x + 1] - c0 - 1);
-        auto bload = [&](int j) -> int64_t { return j <= nchk ? crun[c0 + j] : 0; };
-        auto rload = [&](int64_t i) -> MrRun { MrRun r{0, 0, 0}; if (i >= 0 && i < n_runs) r = runs[i]; return r; };
-        int64_t bnd = bload(lane), bnd_next = bload(31 + lane);
-        int cb = 0;
-        int64_t rb = __shfl_sync(0xffffffffu, bnd, 0);
-        MrRun w0 = rload(rb + lane), w1 = rload(rb + 32 + lane), w2 = rload(rb + 64 + lane);
+        pdl_wait();
+    } else if (warp >= W_BPROD) {
+        // ---------------------------------------------------------------- B producers
+        // VPR threads copy a row (16 bytes each), so the 128 threads take RPS rows a step; a
+        // thread's row indices of the next chunk are loaded ahead.  16-byte vector j of K row kc
+        // goes to vector j ^ (kc mod 8) of its 128-byte swizzle row (64-byte rows: j ^ (kc / 2 mod
+        // 4)).  Row-gathering bulk tensor copies (tile::gather4) in their place took 395 against
+        // 193 us for the UY phase of 64 right-hand sides at 40,000 elements: about 90 cycles
+        // per four 128-byte rows.
+        constexpr int VPR = 4 * KP / 16, RPS = 32 * MR_BW / VPR, NST = MR_CW / RPS;
+        const int bt = threadIdx.x - 32 * W_BPROD, brow = bt / VPR, v = bt % VPR;
+        unsigned g = 0;
         bool ok = true;
-        int issued = 0;
-        for (int g = 0; g < nchk && ok; ++g) {
-            if (g - cb >= 31) {
-                cb += 31;
-                bnd = bnd_next;
-                bnd_next = bload(cb + 31 + lane);
-            }
-            const int64_t r0 = __shfl_sync(0xffffffffu, bnd, g - cb), r1 = __shfl_sync(0xffffffffu, bnd, g - cb + 1);
-            while (r0 >= rb + 32) {
-                rb += 32;
-                w0 = w1;
-                w1 = w2;
-                w2 = rload(rb + 64 + lane);
-            }
-            const int64_t i0 = rb + lane, i1 = i0 + 32, i2 = i0 + 64;
-            const bool h0 = i0 >= r0 && i0 < r1, h1 = i1 >= r0 && i1 < r1, h2 = i2 >= r0 && i2 < r1;
-            unsigned bytes = ((h0 ? w0.len : 0) + (h1 ? w1.len : 0) + (h2 ? w2.len : 0)) * (unsigned)KP * 4u;
+        MrTask tn;
+        if (blockIdx.x < ntasks) tn = tasks[blockIdx.x];
+        int nxt[NST];
+        auto load = [&](const MrTask &t, int c) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) bytes += __shfl_xor_sync(0xffffffffu, bytes, o);
-            const int s = g % MR_SS;
-            if (g >= MR_SS && !mr_warp_wait(&s_empty[s], ((g / MR_SS) - 1) & 1, fail)) { ok = false; break; }
-            if (lane == 0) mr_expect_tx(&s_full[s], bytes);   // 0 bytes: the phase completes on the arrival
-            __syncwarp();
-            unsigned char *stg = sS + (size_t)s * SSTAGE;
-            if (h0) mr_bulk(stg + (size_t)w0.dst * KP * 4, xt + w0.src * KP, (unsigned)w0.len * KP * 4u, &s_full[s]);
-            if (h1) mr_bulk(stg + (size_t)w1.dst * KP * 4, xt + w1.src * KP, (unsigned)w1.len * KP * 4u, &s_full[s]);
-            if (h2) mr_bulk(stg + (size_t)w2.dst * KP * 4, xt + w2.src * KP, (unsigned)w2.len * KP * 4u, &s_full[s]);
-            ++issued;
-        }
-        if (*fail && lane == 0) {   // let the copies in flight land before the CTA exits
-            const unsigned g = (unsigned)issued;
-            for (int s = 0; s < MR_SS; ++s) {
-                const unsigned uses = g / MR_SS + (s < (int)(g % MR_SS) ? 1u : 0u);
-                if (uses == 0) continue;
-                const unsigned long long t0 = mr_ns();
-                while (!mr_try(&s_full[s], (uses - 1) & 1) && mr_ns() - t0 < MR_WAIT_NS) {
+            for (int u = 0; u < NST; ++u) nxt[u] = bidx[t.g_off + (int64_t)c * MR_CW + u * RPS + brow];
+        };
+        if (blockIdx.x < ntasks) load(tn, 0);
+        pdl_wait();
+        for (int ti = blockIdx.x; ti < ntasks && ok; ti += gridDim.x) {
+            const MrTask t = tn;
+            const bool more = ti + (int)gridDim.x < ntasks;
+            if (more) tn = tasks[ti + gridDim.x];
+            const int nch = mr_nchunks(t);
+            for (int c = 0; c < nch; ++c, ++g) {
+                int r[NST];
+#pragma unroll
+                for (int u = 0; u < NST; ++u) r[u] = nxt[u];
+                if (c + 1 < nch) load(t, c + 1);
+                else if (more) load(tn, 0);
+                const int w = mr_chunk(t, c).w;
+                const int s = g % MR_SB;
+                if (g >= (unsigned)MR_SB && !mr_warp_wait(&b_empty[s], ((g / MR_SB) - 1) & 1, fail)) { ok = false; break; }
+                const unsigned stage = mr_smem(sB + (size_t)s * BSTAGE);
+#pragma unroll
+                for (int u = 0; u < NST; ++u) {
+                    const int kc = u * RPS + brow;
+                    if (kc < w) {
+                        const int at = v / (ROWB / 16), j = v % (ROWB / 16);
+                        const int sj = ROWB == 128 ? j ^ (kc & 7) : j ^ ((kc >> 1) & 3);
+                        mr_copy16(stage + (unsigned)(at * BATOM + kc * ROWB + sj * 16), x16 + (int64_t)r[u] * 2 * KP + v * 8);
+                    }
                 }
+                mr_copy_arrive(&b_full[s]);
             }
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");   // the copies in flight land before the CTA exits
     } else if (warp == W_MMA) {
         // ---------------------------------------------------------------- MMA issuer
+        pdl_wait();
         if (lane == 0) {
             // D F32 (bits 4-5 = 1), A and B F16, A K-major, B MN-major (bit 16), M = 128; N = 2 KP
             // for A_hi [B_hi | B_lo] into the adjacent accumulators D1 | D2, N = KP for A_lo B_hi
@@ -439,18 +457,18 @@ __global__ void __launch_bounds__(MR_THREADS, 1)
                         ok = false;
                         break;
                     }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the copied B rows, for the MMA
                     mr_fence_after();
                     const unsigned a0 = mr_smem(sA + (size_t)sa * MR_A_STAGE);
                     const unsigned a1 = mr_smem(sA + (size_t)sa2 * MR_A_STAGE);
-                    const unsigned bst = mr_smem(sB + (size_t)sb * 2 * BSTAGE);
+                    const unsigned bst = mr_smem(sB + (size_t)sb * BSTAGE);
                     const unsigned sbo_a = (unsigned)k.w * 16u;
-                    // descriptors of the chunk's first K step: the B operand's K groups are 2 KP x 16
-                    // bytes apart, its N groups 128; a K step of 16 columns moves A by two core
-                    // matrices (256 bytes) and B by two K groups (64 KP bytes), i.e. the start-address
-                    // field (address / 16, low bits) by 16 and 4 KP.  The N = KP descriptor reads the
-                    // hi half (the first RQ N groups) of the same operand.
-                    uint64_t ah = mr_desc(a0, 128u, sbo_a), al = mr_desc(a1, 128u, sbo_a);
-                    uint64_t bd = mr_desc(bst, (unsigned)KP * 32u, 128u);
+                    // descriptors of the chunk's first K step; a K step of 16 columns moves A by
+                    // two core matrices (256 bytes) and B by 16 K rows (16 ROWB bytes), i.e. the
+                    // start-address field (address / 16, low bits) by 16 and ROWB.  The N = KP MMA
+                    // reads the hi half of the same operand.
+                    uint64_t ah = mr_desc(a0, 128u, sbo_a, 0u), al = mr_desc(a1, 128u, sbo_a, 0u);
+                    uint64_t bd = mr_desc(bst, (unsigned)BATOM, 8u * ROWB, SWZ);
                     const int nk = k.w / 16;
                     for (int kk = 0; kk < nk; ++kk) {
                         mr_mma(d1, ah, bd, idesc2, acc1);
@@ -458,7 +476,7 @@ __global__ void __launch_bounds__(MR_THREADS, 1)
                         if (k.parts == 2) mr_mma(d2, al, bd, idesc1, 1u);
                         ah += 16u;
                         al += 16u;
-                        bd += 4u * KP;
+                        bd += (unsigned)ROWB;
                     }
                     mr_commit(&a_empty[sa]);
                     if (k.parts == 2) mr_commit(&a_empty[sa2]);
@@ -476,83 +494,13 @@ __global__ void __launch_bounds__(MR_THREADS, 1)
             while (!mr_try(&fin, 0) && mr_ns() - t0 < MR_WAIT_NS) {
             }
         }
-    } else if (warp < MR_GW) {
-        // ---------------------------------------------------------------- converters (warp w: chunks w mod 4)
-        unsigned gc = 0;   // chunk index in this CTA's sequence
-        bool ok = true;
-        MrTask tn;
-        if (blockIdx.x < ntasks) tn = tasks[blockIdx.x];
-        for (int ti = blockIdx.x; ti < ntasks && ok; ti += gridDim.x) {
-            const MrTask t = tn;
-            if (ti + (int)gridDim.x < ntasks) tn = tasks[ti + gridDim.x];
-            const int nch = mr_nchunks(t);
-            for (int c = 0; c < nch; ++c, ++gc) {
-                if ((int)(gc % MR_GW) != warp) continue;
-                const MrChunk k = mr_chunk(t, c);
-                const int sb = gc % MR_SB, ss = gc % MR_SS;
-                if (gc >= MR_SB && !mr_warp_wait(&b_empty[sb], ((gc / MR_SB) - 1) & 1, fail)) { ok = false; break; }
-                if (!mr_warp_wait(&s_full[ss], (gc / MR_SS) & 1, fail)) { ok = false; break; }
-                __syncwarp();
-                const float *stg = reinterpret_cast<const float *>(sS + (size_t)ss * SSTAGE);
-                unsigned char *bst = sB + (size_t)sb * 2 * BSTAGE;
-                // Vector (kc, rq): K row kc = 8 kg + kr, right-hand sides 8 rq .. 8 rq + 7, one
-                // 16-byte row of core matrix (kg, rq).  A 16-byte shared-memory access is served
-                // eight lanes at a time; those eight lanes take the eight K rows kr = p of one kg
-                // (their stores hit eight different 16-byte bank groups of a core-matrix row
-                // set) with right-hand-side blocks rq = base + off(p) and the two float4 halves
-                // of their staging row read in the order h(p), 1 - h(p): the staging word
-                // kc KP + 8 rq + 4 h lies in bank group (kc KP / 4 + 2 rq + h) mod 8, and off,
-                // h are chosen so that these eight groups differ as well.
-                constexpr int RQ = KP / 8;
-                constexpr bool KP_MOD32 = (KP / 4) % 8 == 0;   // KP = 32, 64: kc KP / 4 = 0 mod 8
-                const int p = lane & 7;
-                const int h = KP_MOD32 ? (p & 1) : ((p >> 1) & 1);
-                const int roff = KP_MOD32 ? (p >> 1) : (p >> 2);
-                const int npairs = (k.w / 8) * RQ;
-                for (int u = lane >> 3; u < npairs; u += 4) {
-                    const int kg = u / RQ, base = u - kg * RQ;
-                    const int rq = base + roff < RQ ? base + roff : base + roff - RQ;
-                    const int kr = p;
-                    const int kc = 8 * kg + kr, col = k.col0 + kc;
-                    // padding at the end of the dense and of the factor segment: zeros (not copied)
-                    const bool pad = col < t.kd ? col >= t.nd_real : col - t.kd >= t.nl_real;
-                    __align__(16) __half hi[8], lo[8];
-                    if (!pad) {
-                        const float *src = stg + kc * KP + 8 * rq, *scl = s_scale + 8 * rq;
-                        const float4 xa = *reinterpret_cast<const float4 *>(src + 4 * h);
-                        const float4 xb = *reinterpret_cast<const float4 *>(src + 4 - 4 * h);
-                        const float4 sa = *reinterpret_cast<const float4 *>(scl + 4 * h);
-                        const float4 sb = *reinterpret_cast<const float4 *>(scl + 4 - 4 * h);
-                        const float4 x0 = h ? xb : xa, x1 = h ? xa : xb;
-                        const float4 s0 = h ? sb : sa, s1 = h ? sa : sb;
-                        const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-                        const float ss[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const float b = xs[q] * ss[q];
-                            hi[q] = __float2half_rn(b);
-                            lo[q] = __float2half_rn((b - __half2float(hi[q])) * 2048.0f);
-                        }
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) hi[q] = lo[q] = __float2half_rn(0.0f);
-                    }
-                    // one B operand of N = 2 KP: K group kg holds the hi core matrices (N groups
-                    // 0 .. RQ - 1) and then the lo ones (RQ .. 2 RQ - 1), 128 bytes each
-                    const int off = (kg * 2 * RQ + rq) * 128 + kr * 16;
-                    *reinterpret_cast<uint4 *>(bst + off) = *reinterpret_cast<const uint4 *>(hi);
-                    *reinterpret_cast<uint4 *>(bst + off + RQ * 128) = *reinterpret_cast<const uint4 *>(lo);
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                mr_arrive(&s_empty[ss]);
-                mr_arrive(&b_full[sb]);
-                __syncwarp();
-            }
-        }
     } else {
-        // ---------------------------------------------------------------- epilogue (warps 4-7)
-        const int row = threadIdx.x - 32 * W_EPI;          // 0..127 = TMEM lane = panel row
-        const unsigned lane_base = (unsigned)(32 * (warp & 3)) << 16;
+        // ---------------------------------------------------------------- epilogue (warps 0-3)
+        pdl_wait();
+        if (threadIdx.x < KP) s_inv[threadIdx.x] = 1.0f / mr_phase_scale(vmax, vt, threadIdx.x);
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * MR_GW) : "memory");
+        const int row = threadIdx.x;                       // 0..127 = TMEM lane = panel row
+        const unsigned lane_base = (unsigned)(32 * warp) << 16;
         unsigned nt = 0;
         MrTask tn;
         if (blockIdx.x < ntasks) tn = tasks[blockIdx.x];
@@ -597,10 +545,13 @@ __global__ void __launch_bounds__(MR_THREADS, 1)
             mr_arrive(&acc_empty[ab]);
         }
     }
-    if (threadIdx.x == 0 && s_fail) atomicExch(err, 1);
     mr_fence_before();
     __syncthreads();
     mr_fence_after();
+    if (threadIdx.x == 0 && s_fail) {   // err is host memory
+        *(volatile int *)err = 1;
+        __threadfence_system();
+    }
     if (vt && threadIdx.x < KP && s_tmax[threadIdx.x]) atomicMax(vmax + 64 + threadIdx.x, s_tmax[threadIdx.x]);
     if (warp == W_MMA)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(TCOLS) : "memory");
@@ -611,62 +562,73 @@ constexpr int MR_TILE = 32;   // rows of the shared-memory transpose tiles of th
 // The k inputs (caller's order, component-major, FP64) into [X | X with the dense column
 // scales] in the permuted row order, KP FP32 words per row (right-hand sides k .. KP - 1 zero),
 // and the largest magnitudes per right-hand side into vmax[r] (X) and vmax[128 + r] (scaled X).
-// A tile of 32 consecutive elements of the caller's order, all their components, goes through
-// shared memory: read with consecutive threads on consecutive elements of one component and
-// right-hand side (coalesced), written as whole rows of KP words at the elements' permuted
-// positions (iperm).  The block size is a multiple of KP, so a thread writes one right-hand side
-// throughout and keeps its maxima in registers (one shared and one global atomic per
-// right-hand side and block).
-__global__ void mr_in_kernel(const double *__restrict__ X, const int *__restrict__ iperm, int n, int nin, int k, int KP,
-                             const float *__restrict__ cscale, float *__restrict__ xt, unsigned *__restrict__ vmax) {
-    __shared__ float tile[MR_TILE * 2][MR_KP_MAX + 1];
-    __shared__ unsigned s_m[2][MR_KP_MAX];
-    const int tid = threadIdx.x, nt = blockDim.x;
+// A tile of 32 consecutive elements of the caller's order, one component, goes through shared
+// memory: read with consecutive threads on consecutive elements of one right-hand side
+// (coalesced, a thread's KP / 8 reads in flight together), written as whole rows of KP words at the
+// elements' permuted positions (iperm).  A thread writes one right-hand side throughout and keeps
+// its maxima in registers (one shared and one global atomic per right-hand side and block).
+template <int KP>
+__global__ void __launch_bounds__(256) mr_in_kernel(const double *X, const int *__restrict__ iperm, int n, int nin, int k,
+                                                    const float *__restrict__ cscale, float *xt, unsigned *vmax) {
+    __shared__ float tile[MR_TILE][KP + 1];
+    __shared__ unsigned s_m[2][KP];
+    constexpr int NL = KP * MR_TILE / 256;   // values of a tile per thread
+    const int tid = threadIdx.x;
     const int64_t nx = (int64_t)nin * n;
-    const int trows = MR_TILE * nin;
-    for (int q = tid; q < 2 * MR_KP_MAX; q += nt) s_m[q / MR_KP_MAX][q % MR_KP_MAX] = 0u;
-    __syncthreads();
+    const int64_t ntile = ((int64_t)n + MR_TILE - 1) / MR_TILE * nin;
+    for (int q = tid; q < 2 * KP; q += 256) s_m[q / KP][q % KP] = 0u;
+    pdl_wait();
     float m = 0.0f, mc = 0.0f;
-    const int64_t ntile = ((int64_t)n + MR_TILE - 1) / MR_TILE;
+    const int jl = tid % MR_TILE, rr = tid / MR_TILE;   // reading: element, first right-hand side
+    const int wr = tid % KP, wj = tid / KP;             // writing: right-hand side, first element
     for (int64_t t = blockIdx.x; t < ntile; t += gridDim.x) {
-        const int64_t j0 = t * MR_TILE;
-        __syncthreads();   // the previous tile is written out
-        for (int q = tid; q < trows * KP; q += nt) {
-            const int jl = q % MR_TILE, cr = q / MR_TILE, c = cr % nin, r = cr / nin;
-            const int64_t j = j0 + jl;
-            tile[jl * nin + c][r] = (r < k && j < n) ? (float)X[(int64_t)r * nx + (int64_t)c * n + j] : 0.0f;
+        const int c = (int)(t % nin);
+        const int64_t j0 = t / nin * MR_TILE, j = j0 + jl;
+        double v[NL];
+#pragma unroll
+        for (int u = 0; u < NL; ++u) {
+            const int r = rr + u * (256 / MR_TILE);
+            v[u] = r < k && j < n ? X[(int64_t)r * nx + (int64_t)c * n + j] : 0.0;
         }
+        __syncthreads();   // the previous tile is written out
+#pragma unroll
+        for (int u = 0; u < NL; ++u) tile[jl][rr + u * (256 / MR_TILE)] = (float)v[u];
         __syncthreads();
-        for (int q = tid; q < trows * KP; q += nt) {
-            const int tr = q / KP, r = q - tr * KP, jl = tr / nin, c = tr - jl * nin;
-            const int64_t j = j0 + jl;
-            if (j >= n) break;
-            const int64_t row = (int64_t)iperm[j] * nin + c;
-            const float v = tile[tr][r], vc = v * cscale[row];
-            xt[row * KP + r] = v;             // X, the V^T phase's input
-            xt[nx * KP + row * KP + r] = vc;  // X with the row's dense column scale, the near field's input
-            const float a = fabsf(v), ac = fabsf(vc);
+#pragma unroll
+        for (int u = 0; u < NL; ++u) {
+            const int e = wj + u * (256 / KP);
+            if (j0 + e >= n) break;
+            const int64_t row = (int64_t)iperm[j0 + e] * nin + c;
+            const float x = tile[e][wr], xc = x * cscale[row];
+            xt[row * KP + wr] = x;              // X, the V^T phase's input
+            xt[(nx + row) * KP + wr] = xc;      // X with the row's dense column scale, the near field's input
+            const float a = fabsf(x), ac = fabsf(xc);
             if (isfinite(a)) m = fmaxf(m, a);
             if (isfinite(ac)) mc = fmaxf(mc, ac);
         }
     }
-    if (m > 0.0f) atomicMax(&s_m[0][tid % KP], __float_as_uint(m));
-    if (mc > 0.0f) atomicMax(&s_m[1][tid % KP], __float_as_uint(mc));
+    if (m > 0.0f) atomicMax(&s_m[0][wr], __float_as_uint(m));
+    if (mc > 0.0f) atomicMax(&s_m[1][wr], __float_as_uint(mc));
     __syncthreads();
-    for (int r = tid; r < KP; r += nt) {
-        if (s_m[0][r]) atomicMax(vmax + r, s_m[0][r]);
-        if (s_m[1][r]) atomicMax(vmax + 128 + r, s_m[1][r]);
+    if (tid < KP) {
+        if (s_m[0][tid]) atomicMax(vmax + tid, s_m[0][tid]);
+        if (s_m[1][tid]) atomicMax(vmax + 128 + tid, s_m[1][tid]);
     }
 }
 
 // t of the V^T row tiles cut along K: the sum of their slices' partial rows, in slice order
-// (deterministic), and its largest magnitude per right-hand side into vmax[64 + r].
-__global__ void mr_reduce_kernel(const MrSplit *__restrict__ sp, int KP, float *xt, unsigned *vmax) {
-    __shared__ unsigned s_m[MR_KP_MAX];
+// (deterministic), and its largest magnitude per right-hand side into vmax[64 + r].  MR_RED_ROWS rows
+// of a tile per block, so that the few tiles of the wide groups spread over the chip.
+constexpr int MR_RED_ROWS = 16;
+template <int KP>
+__global__ void __launch_bounds__(256) mr_reduce_kernel(const MrSplit *__restrict__ sp, float *xt, unsigned *vmax) {
+    __shared__ unsigned s_m[KP];
     const MrSplit S = sp[blockIdx.x];
     if (threadIdx.x < KP) s_m[threadIdx.x] = 0u;
     __syncthreads();
-    for (int e = threadIdx.x; e < S.rows * KP; e += blockDim.x) {
+    pdl_wait();
+    const int r1 = min(S.rows, ((int)blockIdx.y + 1) * MR_RED_ROWS);
+    for (int e = (int)blockIdx.y * MR_RED_ROWS * KP + (int)threadIdx.x; e < r1 * KP; e += 256) {
         const int r = e / KP, j = e - r * KP;
         float v = 0.0f;
         for (int q = 0; q < S.nsl; ++q) v += xt[(S.p_row + (int64_t)q * MR_ROWS + r) * KP + j];
@@ -679,30 +641,39 @@ __global__ void mr_reduce_kernel(const MrSplit *__restrict__ sp, int KP, float *
 }
 
 // The permuted outputs (KP FP32 words per row) into the caller's order, component-major, FP64:
-// a tile of 32 consecutive elements of the caller's order, all their components, read as whole
-// rows at the elements' permuted positions and written with consecutive threads on consecutive
-// elements of one component and right-hand side (coalesced).
-__global__ void mr_out_kernel(const float *__restrict__ yp, const int *__restrict__ iperm, int n, int nout, int k, int KP,
-                              double *__restrict__ Y) {
-    __shared__ float tile[MR_TILE * 3][MR_KP_MAX + 1];
-    const int tid = threadIdx.x, nt = blockDim.x;
+// a tile of 32 consecutive elements of the caller's order, one component, read as whole rows at
+// the elements' permuted positions (a thread's reads in flight together) and written with
+// consecutive threads on consecutive elements of one right-hand side (coalesced).
+template <int KP>
+__global__ void __launch_bounds__(256) mr_out_kernel(const float *yp, const int *__restrict__ iperm, int n, int nout, int k,
+                                                     double *Y) {
+    __shared__ float tile[MR_TILE][KP + 1];
+    constexpr int NL = KP * MR_TILE / 256;
+    const int tid = threadIdx.x;
     const int64_t ny = (int64_t)nout * n;
-    const int trows = MR_TILE * nout;
-    const int64_t ntile = ((int64_t)n + MR_TILE - 1) / MR_TILE;
+    const int64_t ntile = ((int64_t)n + MR_TILE - 1) / MR_TILE * nout;
+    const int jl = tid % MR_TILE, rr = tid / MR_TILE;   // writing
+    const int wr = tid % KP, wj = tid / KP;             // reading
+    pdl_wait();
     for (int64_t t = blockIdx.x; t < ntile; t += gridDim.x) {
-        const int64_t j0 = t * MR_TILE;
+        const int c = (int)(t % nout);
+        const int64_t j0 = t / nout * MR_TILE, j = j0 + jl;
+        float v[NL];
+#pragma unroll
+        for (int u = 0; u < NL; ++u) {
+            const int e = wj + u * (256 / KP);
+            v[u] = j0 + e < n ? yp[((int64_t)iperm[j0 + e] * nout + c) * KP + wr] : 0.0f;
+        }
         __syncthreads();   // the previous tile is written out
-        for (int q = tid; q < trows * KP; q += nt) {
-            const int tr = q / KP, r = q - tr * KP, jl = tr / nout, c = tr - jl * nout;
-            const int64_t j = j0 + jl;
-            tile[tr][r] = j < n ? yp[((int64_t)iperm[j] * nout + c) * KP + r] : 0.0f;
-        }
+#pragma unroll
+        for (int u = 0; u < NL; ++u) tile[wj + u * (256 / KP)][wr] = v[u];
         __syncthreads();
-        for (int q = tid; q < trows * k; q += nt) {
-            const int jl = q % MR_TILE, cr = q / MR_TILE, c = cr % nout, r = cr / nout;
-            const int64_t j = j0 + jl;
-            if (j < n) Y[(int64_t)r * ny + (int64_t)c * n + j] = (double)tile[jl * nout + c][r];
-        }
+        if (j < n)
+#pragma unroll
+            for (int u = 0; u < NL; ++u) {
+                const int r = rr + u * (256 / MR_TILE);
+                if (r < k) Y[(int64_t)r * ny + (int64_t)c * n + j] = (double)tile[jl][r];
+            }
     }
 }
 
@@ -794,26 +765,19 @@ int64_t mr_task_bytes(const MrTask &t) {
 }
 
 template <int KP> const void *mr_fn() { return (const void *)mr_kernel<KP>; }
-const void *mr_fn_for(int kp) {
-    switch (kp) {
-        case 16: return mr_fn<16>();
-        case 32: return mr_fn<32>();
-        case 48: return mr_fn<48>();
-        default: return mr_fn<64>();
-    }
-}
-int mr_smem_bytes(int kp) { return mr_stages_a(kp) * MR_A_STAGE + MR_SB * 2 * MR_CW * kp * 2 + MR_SS * MR_CW * kp * 4; }
+const void *mr_fn_for(int kp) { return kp == 16 ? mr_fn<16>() : (kp == 32 ? mr_fn<32>() : mr_fn<64>()); }
+int mr_smem_bytes(int kp) { return mr_stages_a(kp) * MR_A_STAGE + mr_stages_b(kp) * MR_CW * kp * 4; }
 
 }  // namespace
 
 void multi_free(hbi_handle *h) {
     MultiRhs *m = h->mr;
     if (!m) return;
-    void *ptrs[] = {m->d_panels, m->d_vt, m->d_uy, m->d_split, m->d_runs[0], m->d_runs[1], m->d_crun[0], m->d_crun[1],
-                    m->d_cta[0], m->d_cta[1], m->d_cscale, m->d_iperm, m->d_rowscale, m->d_xt, m->d_yp, m->d_vmax,
-                    m->d_err};
+    void *ptrs[] = {m->d_panels, m->d_vt, m->d_uy, m->d_split, m->d_bidx, m->d_cscale, m->d_iperm, m->d_rowscale,
+                    m->d_xt, m->d_yp, m->d_x16, m->d_vmax};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+    if (m->h_err) cudaFreeHost(m->h_err);
     delete m;
     h->mr = nullptr;
 }
@@ -923,8 +887,6 @@ hbi_status pack_multi(hbi_handle *h, std::vector<Block> &blocks, const std::vect
                 P.t.kreal = (int)w;
                 P.t.lo = 0;
                 P.t.partial = nsl > 1;
-                P.t.nd_real = 0;
-                P.t.nl_real = (int)w;
                 P.src0 = (int)vrows.size();
                 P.nsrc = rows;
                 for (int i = 0; i < rows; ++i) vrows.push_back(MrRowSrc{rs[q + i].v + c0, rs[q + i].inv_scale});
@@ -1003,8 +965,6 @@ hbi_status pack_multi(hbi_handle *h, std::vector<Block> &blocks, const std::vect
             P.t.kl = (int)kl;
             P.t.kreal = (int)(kd + kl);
             P.t.lo = lo;
-            P.t.nd_real = (int)Cd;
-            P.t.nl_real = (int)Cl;
             P.src0 = (int)terms.size();
             P.nsrc = (int)ut.size();
             for (const MrTerm &T0 : ut) {
@@ -1050,31 +1010,30 @@ hbi_status pack_multi(hbi_handle *h, std::vector<Block> &blocks, const std::vect
     HBI_CUDA_TRY(cudaGetLastError());
     HBI_CUDA_TRY(cudaDeviceSynchronize());
 
-    // gather runs: per chunk, the maximal ranges of consecutive xt rows landing on consecutive
-    // chunk columns (padding columns are left out and read as zeros)
-    auto add_runs = [&](const MrTask &t, int phase) {
-        std::vector<MrRun> &runs = M->h_runs[phase];
-        std::vector<int64_t> &crun = M->h_crun[phase];
-        M->h_cfirst[phase].push_back((int64_t)crun.size());
+    // B row indices: MR_CW per chunk of every task, padding columns at the row of zeros after T
+    // (the row tiles of one leaf row unit share theirs)
+    std::vector<int> bidx;
+    int64_t last_gather = -1, last_off = 0;
+    auto add_rows = [&](MrTask &t, int phase) {
+        const int64_t gather = t.g_off;   // V^T: first X row of the slice; UY: the unit's gather list
+        if (phase == 1 && gather == last_gather) {
+            t.g_off = last_off;
+            return;
+        }
+        t.g_off = (int64_t)bidx.size();
+        if (phase == 1) { last_gather = gather; last_off = t.g_off; }
         const int nchd = (t.kd + MR_CW - 1) / MR_CW, nch = nchd + (t.kl + MR_CW - 1) / MR_CW;
         for (int c = 0; c < nch; ++c) {
-            crun.push_back((int64_t)runs.size());
             const int col0 = c < nchd ? c * MR_CW : t.kd + (c - nchd) * MR_CW;
-            const int w = c < nchd ? std::min(MR_CW, t.kd - col0) : std::min(MR_CW, t.kd + t.kl - col0);
-            const size_t first = runs.size();
-            for (int kc = 0; kc < w; ++kc) {
+            const int end = c < nchd ? t.kd : t.kd + t.kl;
+            for (int kc = 0; kc < MR_CW; ++kc) {
                 const int col = col0 + kc;
-                int64_t j;
-                if (phase == 0) j = col < t.kreal ? t.g_off + col : -1;   // V^T: X rows of the group
-                else j = gidx[t.g_off + col];
-                if (j < 0) continue;
-                if (runs.size() > first && runs.back().src + runs.back().len == j && runs.back().dst + runs.back().len == kc)
-                    ++runs.back().len;
-                else
-                    runs.push_back(MrRun{j, 1, kc});
+                int64_t j = -1;
+                if (phase == 0) j = col < t.kreal ? gather + col : -1;
+                else if (col < end) j = gidx[gather + col];
+                bidx.push_back(j >= 0 ? (int)j : (int)(2 * M->nx + tcount));
             }
         }
-        crun.push_back((int64_t)runs.size());
     };
     std::vector<MrTask> tv, tu;
     for (auto &P : pvt) tv.push_back(P.t);
@@ -1082,14 +1041,16 @@ hbi_status pack_multi(hbi_handle *h, std::vector<Block> &blocks, const std::vect
     // V^T tasks largest first (they are independent); UY tasks in tree order, so that the
     // units running at the same time share far-field t entries in L2
     std::stable_sort(tv.begin(), tv.end(), [](const MrTask &a, const MrTask &b) { return mr_task_bytes(a) > mr_task_bytes(b); });
-    for (const MrTask &t : tv) add_runs(t, 0);
-    for (const MrTask &t : tu) add_runs(t, 1);
+    for (MrTask &t : tv) add_rows(t, 0);
+    for (MrTask &t : tu) add_rows(t, 1);
     M->n_vt = (int)tv.size();
     M->n_uy = (int)tu.size();
     M->n_split = (int)splits.size();
     if ((st = mr_upload(&M->d_vt, tv)) || (st = mr_upload(&M->d_uy, tu)) || (st = mr_upload(&M->d_split, splits)) ||
-        (st = mr_upload(&M->d_rowscale, rowscale)))
+        (st = mr_upload(&M->d_rowscale, rowscale)) || (st = mr_upload(&M->d_bidx, bidx)))
         return st;
+    HBI_CUDA_TRY(cudaMallocHost((void **)&M->h_err, sizeof(int)));
+    *M->h_err = 0;
     M->bytes_panels_alg = alg;
     M->vec_bytes_per_rhs = 4 * (M->nx + 2 * tcount + (int64_t)nout * n);
     M->flops_per_rhs = flops;
@@ -1098,138 +1059,117 @@ hbi_status pack_multi(hbi_handle *h, std::vector<Block> &blocks, const std::vect
 }
 
 namespace {
-// The B gather runs of phase p in the order the CTAs of a grid of g take their chunks: CTA b
-// takes tasks b, b + g, ...; its chunk boundaries are d_crun[d_cta[b] ...], one more than its
-// chunks, and index the reordered runs.
-hbi_status mr_layout(MultiRhs *M, int p, int ntasks, int g) {
-    const std::vector<int64_t> &cf = M->h_cfirst[p], &hc = M->h_crun[p];
-    const std::vector<MrRun> &hr = M->h_runs[p];
-    std::vector<MrRun> runs;
-    std::vector<int64_t> crun, cta;
-    runs.reserve(hr.size());
-    crun.reserve(hc.size() + g);
-    for (int b = 0; b < g; ++b) {
-        cta.push_back((int64_t)crun.size());
-        for (int ti = b; ti < ntasks; ti += g) {
-            const int64_t f = cf[ti], e = ti + 1 < ntasks ? cf[ti + 1] : (int64_t)hc.size();
-            for (int64_t c = f; c + 1 < e; ++c) {
-                crun.push_back((int64_t)runs.size());
-                runs.insert(runs.end(), hr.begin() + hc[c], hr.begin() + hc[c + 1]);
-            }
-        }
-        crun.push_back((int64_t)runs.size());
-    }
-    cta.push_back((int64_t)crun.size());
-    if (M->d_runs[p]) cudaFree(M->d_runs[p]);
-    if (M->d_crun[p]) cudaFree(M->d_crun[p]);
-    if (M->d_cta[p]) cudaFree(M->d_cta[p]);
-    M->d_runs[p] = nullptr; M->d_crun[p] = M->d_cta[p] = nullptr;
-    hbi_status st;
-    if ((st = mr_upload(&M->d_runs[p], runs)) || (st = mr_upload(&M->d_crun[p], crun)) ||
-        (st = mr_upload(&M->d_cta[p], cta)))
-        return st;
-    return HBI_OK;
-}
-
 hbi_status mr_prepare(hbi_handle *h, int kp) {
     MultiRhs *M = h->mr;
+    const int64_t rows16 = 2 * M->nx + M->n_t + 1;
     if (M->kp_cap < kp) {
         if (M->d_xt) cudaFree(M->d_xt);
         if (M->d_yp) cudaFree(M->d_yp);
+        if (M->d_x16) cudaFree(M->d_x16);
         M->d_xt = M->d_yp = nullptr;
-        M->kp_cap = 0;
-        // xt rows: X, X scaled per row for the near field, T, partial rows of cut V^T tiles
+        M->d_x16 = nullptr;
+        M->kp_cap = M->row_kp = 0;
+        // xt rows: X, X scaled per row for the near field, T, partial rows of cut V^T tiles; x16
+        // rows: the first three, split, and one of zeros
         HBI_ALLOC_TRY(&M->d_xt, (size_t)(2 * M->nx + M->n_t + M->n_prow) * kp * sizeof(float));
         HBI_ALLOC_TRY(&M->d_yp, (size_t)h->nout * h->n * kp * sizeof(float));
+        HBI_ALLOC_TRY(&M->d_x16, (size_t)rows16 * 2 * kp * sizeof(__half));
         M->kp_cap = kp;
     }
-    if (!M->d_vmax) {
-        HBI_ALLOC_TRY(&M->d_vmax, 192 * sizeof(unsigned));
-        HBI_ALLOC_TRY(&M->d_err, sizeof(int));
-        HBI_CUDA_TRY(cudaMemset(M->d_err, 0, sizeof(int)));
-    }
-    const void *fn = mr_fn_for(kp);
-    const int smem = mr_smem_bytes(kp);
-    HBI_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    HBI_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    // CTAs per SM from shared memory, registers and tensor memory (each CTA holds 4 kp columns,
-    // two accumulators, rounded up to a power of two, of the SM's 512)
-    int dev = 0, sms = 0, smem_sm = 0, resv = 0, regs_sm = 0;
-    HBI_CUDA_TRY(cudaGetDevice(&dev));
-    HBI_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    HBI_CUDA_TRY(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
-    HBI_CUDA_TRY(cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev));
-    HBI_CUDA_TRY(cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev));
-    cudaFuncAttributes fa;
-    HBI_CUDA_TRY(cudaFuncGetAttributes(&fa, fn));
-    const int by_smem = smem_sm / (smem + (int)fa.sharedSizeBytes + resv);
-    const int regs_warp = (fa.numRegs * 32 + 255) / 256 * 256;
-    const int by_regs = regs_sm / (regs_warp * (MR_THREADS / 32));
-    const int tcols = 4 * kp <= 64 ? 64 : (4 * kp <= 128 ? 128 : 256);
-    const int per_sm = std::max(1, std::min(std::min(by_smem, by_regs), 512 / tcols));
-    M->grid = sms * per_sm;
-    if (M->layout_grid != M->grid) {
-        hbi_status st;
-        if ((st = mr_layout(M, 0, M->n_vt, std::max(1, std::min(M->grid, M->n_vt)))) ||
-            (st = mr_layout(M, 1, M->n_uy, std::max(1, std::min(M->grid, M->n_uy)))))
-            return st;
-        M->layout_grid = M->grid;
+    if (!M->d_vmax) HBI_ALLOC_TRY(&M->d_vmax, 192 * sizeof(unsigned));
+    if (M->row_kp != kp) {   // the row length, and with it the place of the row of zeros, goes with kp
+        M->zeroed = 0;
+        const void *fn = mr_fn_for(kp);
+        const int smem = mr_smem_bytes(kp);
+        HBI_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        HBI_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        // CTAs per SM from shared memory, registers and tensor memory (each CTA holds 4 kp columns,
+        // two accumulators, of the SM's 512)
+        int dev = 0, sms = 0, smem_sm = 0, resv = 0, regs_sm = 0;
+        HBI_CUDA_TRY(cudaGetDevice(&dev));
+        HBI_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        HBI_CUDA_TRY(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+        HBI_CUDA_TRY(cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev));
+        HBI_CUDA_TRY(cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev));
+        cudaFuncAttributes fa;
+        HBI_CUDA_TRY(cudaFuncGetAttributes(&fa, fn));
+        const int by_smem = smem_sm / (smem + (int)fa.sharedSizeBytes + resv);
+        const int regs_warp = (fa.numRegs * 32 + 255) / 256 * 256;
+        const int by_regs = regs_sm / (regs_warp * (MR_THREADS / 32));
+        const int per_sm = std::max(1, std::min(std::min(by_smem, by_regs), 512 / (4 * kp)));
+        M->grid = sms * per_sm;
+        M->row_kp = kp;
     }
     return HBI_OK;
 }
 
+// Calls f with kp (16, 32 or 64) as a constant.
+template <typename F> hbi_status mr_dispatch(int kp, F &&f) {
+    if (kp == 16) return f(std::integral_constant<int, 16>());
+    if (kp == 32) return f(std::integral_constant<int, 32>());
+    return f(std::integral_constant<int, 64>());
+}
+
+// phase 0: V^T (split of X, the V^T product, sums of its cut tiles); 1: UY (split of scaled X and T,
+// the row product)
 template <int KP>
 hbi_status mr_launch_phase(hbi_handle *h, int phase, cudaStream_t s) {
     MultiRhs *M = h->mr;
-    const int smem = mr_smem_bytes(KP);
-    if (phase == 0 && M->n_vt)
-        mr_kernel<KP><<<std::min(M->grid, M->n_vt), MR_THREADS, smem, s>>>(
-            M->d_vt, M->n_vt, 1, M->d_panels, M->d_runs[0], (int64_t)M->h_runs[0].size(), M->d_crun[0], M->d_cta[0],
-            M->d_rowscale, M->d_xt, M->d_xt, M->d_vmax, M->d_err);
-    if (phase == 0 && M->n_split)
-        mr_reduce_kernel<<<M->n_split, 256, 0, s>>>(M->d_split, KP, M->d_xt, M->d_vmax);
-    if (phase == 1 && M->n_uy)
-        mr_kernel<KP><<<std::min(M->grid, M->n_uy), MR_THREADS, smem, s>>>(
-            M->d_uy, M->n_uy, 0, M->d_panels, M->d_runs[1], (int64_t)M->h_runs[1].size(), M->d_crun[1], M->d_cta[1],
-            M->d_rowscale, M->d_xt, M->d_yp, M->d_vmax, M->d_err);
-    HBI_CUDA_TRY(cudaGetLastError());
+    const int smem = mr_smem_bytes(KP), sms = std::max(1, h->num_sms);
+    auto split = [&](int vt, int64_t row0, int64_t nrows) {
+        const int64_t blocks = (nrows * (KP / 8) + 255) / 256;
+        return launch_dependent(mr_split_kernel<KP>, (int)std::max<int64_t>(1, std::min<int64_t>(blocks, 8 * sms)), 256, 0,
+                                s, M->d_xt, M->d_vmax, vt, row0, nrows, M->d_x16);
+    };
+    if (phase == 0 && M->n_vt) {
+        HBI_CUDA_TRY(split(1, 0, M->nx));
+        HBI_CUDA_TRY(launch_dependent(mr_kernel<KP>, std::min(M->grid, M->n_vt), MR_THREADS, smem, s, M->d_vt, M->n_vt, 1,
+                                      M->d_panels, M->d_x16, M->d_bidx, M->d_rowscale, M->d_xt, M->d_vmax, M->h_err));
+        if (M->n_split) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)M->n_split, MR_ROWS / MR_RED_ROWS);
+            cfg.blockDim = dim3(256);
+            cfg.stream = s;
+            HBI_CUDA_TRY(cudaLaunchKernelEx(&cfg, mr_reduce_kernel<KP>, (const MrSplit *)M->d_split, M->d_xt, M->d_vmax));
+        }
+    }
+    if (phase == 1 && M->n_uy) {
+        HBI_CUDA_TRY(split(0, M->nx, M->nx + M->n_t));
+        HBI_CUDA_TRY(launch_dependent(mr_kernel<KP>, std::min(M->grid, M->n_uy), MR_THREADS, smem, s, M->d_uy, M->n_uy, 0,
+                                      M->d_panels, M->d_x16, M->d_bidx, M->d_rowscale, M->d_yp, M->d_vmax, M->h_err));
+    }
     return HBI_OK;
 }
 hbi_status mr_phase(hbi_handle *h, int kp, int phase, cudaStream_t s) {
-    switch (kp) {
-        case 16: return mr_launch_phase<16>(h, phase, s);
-        case 32: return mr_launch_phase<32>(h, phase, s);
-        case 48: return mr_launch_phase<48>(h, phase, s);
-        default: return mr_launch_phase<64>(h, phase, s);
-    }
+    return mr_dispatch(kp, [&](auto kc) { return mr_launch_phase<decltype(kc)::value>(h, phase, s); });
 }
 
 // the whole product on `s`, no synchronisation
 hbi_status mr_enqueue(hbi_handle *h, int k, int kp, const double *d_X, double *d_Y, cudaStream_t s) {
     MultiRhs *M = h->mr;
     HBI_CUDA_TRY(cudaMemsetAsync(M->d_vmax, 0, 192 * sizeof(unsigned), s));
-    const int gmax = 8 * std::max(1, h->num_sms);
-    const int g = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)h->n + MR_TILE - 1) / MR_TILE, gmax));
-    // a block size that is a multiple of kp (every thread writes one right-hand side)
-    if (d_X) mr_in_kernel<<<g, kp * (256 / kp), 0, s>>>(d_X, M->d_iperm, h->n, h->nin, k, kp, M->d_cscale, M->d_xt, M->d_vmax);
-    HBI_CUDA_TRY(cudaGetLastError());
-    hbi_status st = mr_phase(h, kp, 0, s);
-    if (st) return st;
-    if ((st = mr_phase(h, kp, 1, s))) return st;
-    if (d_Y) {
-        const int64_t ny = (int64_t)h->nout * h->n;
-        const int g2 = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)h->n + MR_TILE - 1) / MR_TILE, gmax));
-        mr_out_kernel<<<g2, 256, 0, s>>>(M->d_yp, M->d_iperm, h->n, h->nout, k, kp, d_Y);
-        HBI_CUDA_TRY(cudaGetLastError());
+    if (!M->zeroed) {
+        HBI_CUDA_TRY(cudaMemsetAsync(M->d_x16 + (2 * M->nx + M->n_t) * 2 * kp, 0, (size_t)2 * kp * sizeof(__half), s));
+        M->zeroed = 1;
     }
-    return HBI_OK;
+    const int64_t ntile = ((int64_t)h->n + MR_TILE - 1) / MR_TILE, most = 8 * std::max(1, h->num_sms);
+    const int gin = (int)std::min<int64_t>(ntile * h->nin, most), gout = (int)std::min<int64_t>(ntile * h->nout, most);
+    hbi_status st = mr_dispatch(kp, [&](auto kc) -> hbi_status {
+        HBI_CUDA_TRY(launch_dependent(mr_in_kernel<decltype(kc)::value>, gin, 256, 0, s, d_X, M->d_iperm, h->n, h->nin, k,
+                                      M->d_cscale, M->d_xt, M->d_vmax));
+        return HBI_OK;
+    });
+    if (st || (st = mr_phase(h, kp, 0, s)) || (st = mr_phase(h, kp, 1, s))) return st;
+    return mr_dispatch(kp, [&](auto kc) -> hbi_status {
+        HBI_CUDA_TRY(launch_dependent(mr_out_kernel<decltype(kc)::value>, gout, 256, 0, s, M->d_yp, M->d_iperm, h->n,
+                                      h->nout, k, d_Y));
+        return HBI_OK;
+    });
 }
 
 hbi_status mr_check(hbi_handle *h) {
-    int err = 0;
-    HBI_CUDA_TRY(cudaMemcpy(&err, h->mr->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (err) {
-        HBI_CUDA_TRY(cudaMemset(h->mr->d_err, 0, sizeof(int)));
+    if (*(volatile int *)h->mr->h_err) {
+        *h->mr->h_err = 0;
         set_error("a multi-RHS product wait timed out");
         return HBI_ERR_TIMEOUT;
     }
@@ -1243,7 +1183,7 @@ hbi_status mr_args(hbi_handle *h, int k, int &kp) {
         return HBI_ERR_INVALID_ARG;
     }
     if (k < 1 || k > MR_KP_MAX) { set_error("need 1 <= k <= 64 right-hand sides"); return HBI_ERR_INVALID_ARG; }
-    kp = (int)mr_round(k, 16);
+    kp = k <= 16 ? 16 : (k <= 32 ? 32 : 64);
     if (h->num_sms <= 0) {
         int dev = 0;
         HBI_CUDA_TRY(cudaGetDevice(&dev));
