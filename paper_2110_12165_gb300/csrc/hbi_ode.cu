@@ -135,6 +135,7 @@ __global__ void controller_kernel(OdeArgs A) {
 // Accept: y <- y5, slip by the trapezoid of Eq. 16; either way prepare stage 1 of the next
 // attempt (the HMVM input of the current state).
 __global__ void commit_kernel(OdeArgs A) {
+    pdl_wait();
     if (all_stopped(A)) return;
     const int n = A.n;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -435,7 +436,8 @@ __global__ void adj_loss_kernel(OdeArgs A, const double *__restrict__ target, do
 }
 
 // start of a step's reverse sweep: Kbar_s = dt b5_s lambda
-__global__ void adj_init_kernel(OdeArgs A, const double *__restrict__ lam, double *Kbar, double dt) {
+__global__ void adj_init_kernel(OdeArgs A, const double *lam, double *Kbar, double dt) {
+    pdl_wait();
     const int n3 = 3 * A.n;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n3; j += gridDim.x * blockDim.x) {
         const double l = lam[j];
@@ -444,31 +446,38 @@ __global__ void adj_init_kernel(OdeArgs A, const double *__restrict__ lam, doubl
     }
 }
 
-// stage s, first half: the adjoint of the stress rates, as the input of the product with H^T
-__global__ void adj_pre_kernel(OdeArgs A, int s, const double *__restrict__ Kbar, void *axt) {
+// stage s at element i, first half: the adjoint of the stress rates, as the input of the product
+// with H^T
+__device__ __forceinline__ void adj_pre_elem(const OdeArgs &A, int s, int i, const double *Kbar, void *axt) {
     const int n = A.n;
     const double *Y = A.st_Y + (size_t)s * 3 * n, *S = A.st_S + (size_t)s * A.nout * n;
     const double *K = Kbar + (size_t)s * 3 * n;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double AV, BV, AVb, BVb, d0, d1, d2, d3, d4;
-        stress_from(A, i, S + (size_t)A.nout * i, AV, BV);
-        rhs_vjp_elem(A, i, Y[i], Y[n + i], Y[2 * n + i], AV, BV, K[i], K[n + i], K[2 * n + i], 0.0, AVb, BVb, d0,
-                     d1, d2, d3, d4);
-        double o[3];
-        if (A.nout == 1) { o[0] = AVb; }
-        else if (A.nin == 1) { o[0] = AVb; o[1] = BVb; }
-        else { o[0] = A.cr[i] * AVb; o[1] = A.sr[i] * AVb; o[2] = BVb; }
-        for (int c = 0; c < A.nout; ++c) {
-            if (A.acc_double) ((double *)axt)[(size_t)A.nout * i + c] = o[c];
-            else ((float *)axt)[(size_t)A.nout * i + c] = (float)o[c];
-        }
+    double AV, BV, AVb, BVb, d0, d1, d2, d3, d4;
+    stress_from(A, i, S + (size_t)A.nout * i, AV, BV);
+    rhs_vjp_elem(A, i, Y[i], Y[n + i], Y[2 * n + i], AV, BV, K[i], K[n + i], K[2 * n + i], 0.0, AVb, BVb, d0, d1, d2, d3,
+                 d4);
+    double o[3];
+    if (A.nout == 1) { o[0] = AVb; }
+    else if (A.nin == 1) { o[0] = AVb; o[1] = BVb; }
+    else { o[0] = A.cr[i] * AVb; o[1] = A.sr[i] * AVb; o[2] = BVb; }
+    for (int c = 0; c < A.nout; ++c) {
+        if (A.acc_double) ((double *)axt)[(size_t)A.nout * i + c] = o[c];
+        else ((float *)axt)[(size_t)A.nout * i + c] = (float)o[c];
     }
+}
+__global__ void adj_pre_kernel(OdeArgs A, int s, const double *Kbar, void *axt) {
+    pdl_wait();
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += gridDim.x * blockDim.x)
+        adj_pre_elem(A, s, i, Kbar, axt);
 }
 
 // stage s, second half: with the product H^T (adjoint stress rates) in ayp, the adjoint of
-// the stage state; accumulate lambda, the earlier stages' Kbar and the parameter gradients
+// the stage state; accumulate lambda, the earlier stages' Kbar and the parameter gradients.  axt (not
+// nullptr): then stage s - 1's first half, whose input is the element's own (one launch in place of
+// two between the products).
 __global__ void adj_post_kernel(OdeArgs A, int s, const void *ayp, double *lam, double *Kbar, double *gA,
-                                double *gDC, double dt) {
+                                double *gDC, double dt, void *axt) {
+    pdl_wait();
     const int n = A.n;
     const double *Y = A.st_Y + (size_t)s * 3 * n, *S = A.st_S + (size_t)s * A.nout * n;
     const double *K = Kbar + (size_t)s * 3 * n;
@@ -490,11 +499,13 @@ __global__ void adj_post_kernel(OdeArgs A, int s, const void *ayp, double *lam, 
         }
         gA[i] += ab;
         gDC[i] += dcb;
+        if (axt != nullptr) adj_pre_elem(A, s - 1, i, Kbar, axt);
     }
 }
 
 // fixed-step mode: the step size of the next step, always accepted
 __global__ void fixed_dt_kernel(StepCtl *C, double dt) {
+    pdl_wait();
     C->dt = dt; C->dt_used = dt; C->accept_flag = 1;
     C->stop = 0; C->reuse_k0 = 0;
     C->mu_fix = 0;
@@ -646,37 +657,35 @@ hbi_status ode_prep(hbi_handle *h, cudaStream_t s, int vec) {
     return HBI_OK;
 }
 
-// One attempt: 6 x (HMVM + stage), controller, commit.  A rejected attempt leaves y
-// unchanged, so the next attempt skips its first HMVM and reuses k_0.
-// Stage s (0..5, the last with the error maxima) runs inside the UY phase of product s, unit by
-// unit as the unit's rows are written; the products alternate between the input buffers d_xt
-// (even products: prep and commit write it) and d_xt2, so that stage s can write product
-// s+1's input while other CTAs still gather product s's.
-hbi_status ode_attempt(hbi_handle *h, cudaStream_t s, int vec) {
-    OdeArgs A = args(h);
-    const int *stop = &h->d_gctl->stop;
-    const int g = grid_ode(h);
-    if (!vec) {
-        void *xb[2] = {h->d_xt, h->d_xt2};
-        for (int st = 0; st < 6; ++st) {
-            OdeArgs F = A;
-            F.xt = xb[(st + 1) & 1];
-            hbi_status r = hmvm_launch(h, s, st == 0 ? &h->d_gctl->skip0 : stop,
-                                       st == 0 ? h->d_mskip : h->d_mskip + h->n_models, xb[st & 1], &F, st);
-            if (r) return r;
-        }
-        // controller, commit and stop flags in one launch
-        HBI_CUDA_TRY(launch_dependent(commit_ctl_kernel, g, ODE_BLOCK, 0, s, A));
-        return HBI_OK;
-    }
-    // rake-free friction: the same, with its stage functions; then controller, commit, stop
+// The six products of an attempt or a fixed step with their stages.  Stage s (0..5, the last with
+// the error maxima) runs inside the UY phase of product s, unit by unit as the unit's rows are
+// written; the products alternate between the input buffers d_xt (even products: prep and commit
+// write it) and d_xt2, so that stage s can write product s+1's input while other CTAs still
+// gather product s's.  stop0 / stop: the first / the other products do nothing while it is set
+// (stop = nullptr: stop0 for all); mskip: 2 x n_models skip flags, or nullptr.
+static hbi_status stage_products(hbi_handle *h, const OdeArgs &A, const int *stop0, const int *mskip, const int *stop,
+                                 int law, cudaStream_t s) {
     void *xb[2] = {h->d_xt, h->d_xt2};
     for (int st = 0; st < 6; ++st) {
         OdeArgs F = A;
         F.xt = xb[(st + 1) & 1];
-        hbi_status r = hmvm_launch(h, s, st == 0 ? &h->d_gctl->skip0 : stop,
-                                   st == 0 ? h->d_mskip : h->d_mskip + h->n_models, xb[st & 1], &F, st, 2);
+        hbi_status r = hmvm_launch(h, s, st == 0 || !stop ? stop0 : stop,
+                                   mskip && st > 0 ? mskip + h->n_models : mskip, xb[st & 1], &F, st, law);
         if (r) return r;
+    }
+    return HBI_OK;
+}
+
+// One attempt: 6 x (HMVM + stage), controller, commit.  A rejected attempt leaves y
+// unchanged, so the next attempt skips its first HMVM and reuses k_0.
+hbi_status ode_attempt(hbi_handle *h, cudaStream_t s, int vec) {
+    OdeArgs A = args(h);
+    const int g = grid_ode(h);
+    hbi_status r = stage_products(h, A, &h->d_gctl->skip0, h->d_mskip, &h->d_gctl->stop, vec ? 2 : 1, s);
+    if (r) return r;
+    if (!vec) {   // controller, commit and stop flags in one launch
+        HBI_CUDA_TRY(launch_dependent(commit_ctl_kernel, g, ODE_BLOCK, 0, s, A));
+        return HBI_OK;
     }
     controller_kernel<<<1, 256, 0, s>>>(A);
     commit_vec_kernel<<<g, ODE_BLOCK, 0, s>>>(A);
@@ -759,32 +768,28 @@ hbi_status fixed_reset(hbi_handle *h, cudaStream_t s) {
     return HBI_OK;
 }
 
-// one Cash-Karp step of size dt from the prepared state (ys = y, V, x), always accepted
+// one Cash-Karp step of size dt from the prepared state (ys = y, V, x), always accepted; the
+// stages run inside the products' UY launches as in ode_attempt
 hbi_status fixed_step(hbi_handle *h, const OdeArgs &A, double dt, cudaStream_t s) {
-    const int g = grid_for(h);
-    fixed_dt_kernel<<<1, 1, 0, s>>>(h->d_ctl, dt);
-    for (int st = 0; st < 6; ++st) {
-        hbi_status r = hmvm_launch(h, s, &h->d_gctl->stop);
-        if (r) return r;
-        if (st < 5) stage_kernel<<<g, 256, 0, s>>>(A, st);
-        else final_kernel<<<(h->n + 255) / 256, 256, 0, s>>>(A);
-    }
-    commit_kernel<<<g, 256, 0, s>>>(A);
-    HBI_CUDA_TRY(cudaGetLastError());
+    const int g = grid_ode(h);
+    HBI_CUDA_TRY(launch_dependent(fixed_dt_kernel, 1, 1, 0, s, h->d_ctl, dt));
+    hbi_status r = stage_products(h, A, &h->d_gctl->stop, nullptr, nullptr, 1, s);
+    if (r) return r;
+    HBI_CUDA_TRY(launch_dependent(commit_kernel, g, ODE_BLOCK, 0, s, A));
     return HBI_OK;
 }
 
 // reverse sweep of one step whose stage data are stored (st_Y, st_S); lambda in d_lam
 hbi_status reverse_step(hbi_handle *h, const OdeArgs &A, double dt, cudaStream_t s) {
-    const int g = grid_for(h);
-    adj_init_kernel<<<g, 256, 0, s>>>(A, h->d_lam, h->d_Kbar, dt);
+    const int g = grid_ode(h);
+    HBI_CUDA_TRY(launch_dependent(adj_init_kernel, grid_for(h), 256, 0, s, A, h->d_lam, h->d_Kbar, dt));
+    HBI_CUDA_TRY(launch_dependent(adj_pre_kernel, g, ODE_BLOCK, 0, s, A, 5, h->d_Kbar, h->adj->d_xt));
     for (int st = 5; st >= 0; --st) {
-        adj_pre_kernel<<<g, 256, 0, s>>>(A, st, h->d_Kbar, h->adj->d_xt);
         hbi_status r = hmvm_launch(h->adj, s, nullptr);
         if (r) return r;
-        adj_post_kernel<<<g, 256, 0, s>>>(A, st, h->adj->d_yp, h->d_lam, h->d_Kbar, h->d_gA, h->d_gDC, dt);
+        HBI_CUDA_TRY(launch_dependent(adj_post_kernel, g, ODE_BLOCK, 0, s, A, st, h->adj->d_yp, h->d_lam, h->d_Kbar,
+                                      h->d_gA, h->d_gDC, dt, st > 0 ? h->adj->d_xt : nullptr));
     }
-    HBI_CUDA_TRY(cudaGetLastError());
     return HBI_OK;
 }
 }  // namespace
@@ -879,7 +884,7 @@ hbi_status ode_rhs_vjp(hbi_handle *h, const double *d_v, double *d_ybar, double 
     HBI_CUDA_TRY(cudaMemsetAsync(h->d_gDC, 0, n * sizeof(double), s));
     adj_pre_kernel<<<g, 256, 0, s>>>(A, 0, h->d_Kbar, h->adj->d_xt);
     if ((st = hmvm_launch(h->adj, s, nullptr))) return st;
-    adj_post_kernel<<<g, 256, 0, s>>>(A, 0, h->adj->d_yp, h->d_lam, h->d_Kbar, h->d_gA, h->d_gDC, 0.0);
+    adj_post_kernel<<<g, 256, 0, s>>>(A, 0, h->adj->d_yp, h->d_lam, h->d_Kbar, h->d_gA, h->d_gDC, 0.0, nullptr);
     scatter_state_kernel<<<g, 256, 0, s>>>(h->d_lam, h->d_perm, h->n, 3, d_ybar);
     if (d_grad_a) scatter_state_kernel<<<g, 256, 0, s>>>(h->d_gA, h->d_perm, h->n, 1, d_grad_a);
     if (d_grad_dc) scatter_state_kernel<<<g, 256, 0, s>>>(h->d_gDC, h->d_perm, h->n, 1, d_grad_dc);
