@@ -60,7 +60,7 @@ struct AcaOut { int rank, status; };
 // or column needs one of the pair's n_out rows or n_in columns but evaluates the pair, and its
 // last warp is mostly idle, so 24 rows and columns of a 40 x 40 block cost twice its 1,600 pairs.
 // With one 256-thread CTA (182 registers, one per SM) for every block, in partition order: 282
-// ms for the 9,086 blocks of a 20,022-element fault; so 170 ms one class
+// ms for the 9,086 blocks of a 20,022-element fault; so 134 ms one class
 // after the other, less side by side.
 constexpr int ACA_DENSE = 20;
 
@@ -112,16 +112,32 @@ __device__ double block_sum(double v, double *sv) {
 // residual row moves on to the first unused row; stop once |u_k||v_k| <= eps ||S_k||_F
 // (Frobenius norm of the approximant updated recursively).  Reaching the rank cap
 // floor(m n / (m + n)) marks the block for dense storage.
-// FULL: the block's entries are evaluated first, into `full` (row-major, nc columns).
+// FULL: the block's entries are evaluated first, into `full` (row-major, nc columns).  Otherwise, with
+// `kept` not null, the rows (columns) that an evaluated element pair gives beside the one wanted are
+// kept for the first ACA_KEEP elements on either side: about 30 % of the pivots meet an element
+// again (21 and 25 distinct elements among the 32 pivots of a 128 x 128 block).
+constexpr int ACA_KEEP = 32;
+__host__ __device__ inline int64_t aca_keep_words(int m, int nc, int tau, int sig, int nout, int nin) {
+    // rows kept, columns kept, then a slot number per element and side
+    return (int64_t)ACA_KEEP * ((nout - 1) * nc + (nin - 1) * m) + ((int64_t)tau + sig + 3) / 4;
+}
 template <bool HALF, int THREADS, bool FULL>
-__device__ void aca_block(const EntryGeo &g, const AcaJob &jb, AcaOut *out, double eps, double *full) {
+__device__ void aca_block(const EntryGeo &g, const AcaJob &jb, AcaOut *out, double eps, double *full, double *kept) {
     constexpr int ACA_WARPS = THREADS / 32;
+    __shared__ unsigned char s_rcomp[ACA_KEEP];   // the component a row slot was opened with
+    double *const krow = kept, *const kcol = kept + (int64_t)ACA_KEEP * (g.nout - 1) * jb.nc;
+    short *const rslot = reinterpret_cast<short *>(kcol + (int64_t)ACA_KEEP * (g.nin - 1) * jb.m);
+    short *const cslot = rslot + jb.tau_size;
+    const bool keep = !FULL && kept != nullptr;
+    int nrs = 0, ncs = 0;   // slots in use (the same in every thread)
     __shared__ double sv[ACA_WARPS];
     __shared__ int si[ACA_WARPS];
     __shared__ double s_cross[ACA_WARPS];
     const int m = jb.m, nc = jb.nc;
     unsigned char *urow = jb.flags, *ucol = jb.flags + m;
     for (int k = threadIdx.x; k < m + nc; k += blockDim.x) jb.flags[k] = 0;
+    if (keep)
+        for (int k = threadIdx.x; k < jb.tau_size + jb.sig_size; k += blockDim.x) rslot[k] = -1;
     bool singular = false;
     if (FULL) {
         const int np = jb.tau_size * jb.sig_size;
@@ -149,13 +165,25 @@ __device__ void aca_block(const EntryGeo &g, const AcaJob &jb, AcaOut *out, doub
         // residual row i -> V[:, k]
         double *vk = jb.V + (size_t)k * nc;
         {
-            const int ie = jb.tau_start + i / g.nout, co = i % g.nout;
+            const int il = i / g.nout, ie = jb.tau_start + il, co = i % g.nout;
+            // a kept row (slot >= 0, not the component it was opened with), or one to keep (open >= 0)
+            const int slot = keep && g.nout > 1 ? rslot[il] : -1;
+            const int open = keep && g.nout > 1 && slot < 0 && nrs < ACA_KEEP ? nrs : -1;
+            const int first = slot >= 0 ? s_rcomp[slot] : co;
+            const double *from = krow + ((int64_t)slot * (g.nout - 1) + (co < first ? co : co - 1)) * nc;
             for (int jj = threadIdx.x; jj < jb.sig_size; jj += blockDim.x) {
                 double E[3][2];
-                if (!FULL && !pair_op<HALF>(g, ie, jb.sig_start + jj, E)) singular = true;
+                if (!FULL && slot < 0) {
+                    if (!pair_op<HALF>(g, ie, jb.sig_start + jj, E)) singular = true;
+                    if (open >= 0)
+                        for (int a = 0; a < g.nout; ++a)
+                            if (a != co)
+                                for (int c = 0; c < g.nin; ++c)
+                                    krow[((int64_t)open * (g.nout - 1) + (a < co ? a : a - 1)) * nc + jj * g.nin + c] = E[a][c];
+                }
                 for (int c = 0; c < g.nin; ++c) {
                     const int J = jj * g.nin + c;
-                    double val = FULL ? full[(size_t)i * nc + J] : E[co][c];
+                    double val = FULL ? full[(size_t)i * nc + J] : (slot >= 0 ? from[J] : E[co][c]);
                     for (int l = 0; l < k; ++l) val -= jb.U[(size_t)l * m + i] * jb.V[(size_t)l * nc + J];
                     vk[J] = val;
                 }
@@ -163,6 +191,14 @@ __device__ void aca_block(const EntryGeo &g, const AcaJob &jb, AcaOut *out, doub
         }
         __syncthreads();
         if (threadIdx.x == 0) urow[i] = 1;
+        if (keep && g.nout > 1 && rslot[i / g.nout] < 0 && nrs < ACA_KEEP) {   // the row's element has its slot
+            __syncthreads();   // every thread has read the slot number
+            if (threadIdx.x == 0) {
+                rslot[i / g.nout] = (short)nrs;
+                s_rcomp[nrs] = (unsigned char)(i % g.nout);
+            }
+            ++nrs;
+        }
         double best;
         int j;
         {
@@ -195,13 +231,20 @@ __device__ void aca_block(const EntryGeo &g, const AcaJob &jb, AcaOut *out, doub
         // residual column j -> U[:, k]
         double *uk = jb.U + (size_t)k * m;
         {
-            const int je = jb.sig_start + j / g.nin, ci = j % g.nin;
+            const int jl = j / g.nin, je = jb.sig_start + jl, ci = j % g.nin;
+            const int slot = keep && g.nin > 1 ? cslot[jl] : -1;
+            const int open = keep && g.nin > 1 && slot < 0 && ncs < ACA_KEEP ? ncs : -1;
+            const double *from = kcol + (int64_t)slot * m;   // n_in = 2: the other component
             for (int ii = threadIdx.x; ii < jb.tau_size; ii += blockDim.x) {
                 double E[3][2];
-                if (!FULL && !pair_op<HALF>(g, jb.tau_start + ii, je, E)) singular = true;
+                if (!FULL && slot < 0) {
+                    if (!pair_op<HALF>(g, jb.tau_start + ii, je, E)) singular = true;
+                    if (open >= 0)
+                        for (int a = 0; a < g.nout; ++a) kcol[(int64_t)open * m + ii * g.nout + a] = E[a][1 - ci];
+                }
                 for (int a = 0; a < g.nout; ++a) {
                     const int I = ii * g.nout + a;
-                    double val = FULL ? full[(size_t)I * nc + j] : E[a][ci];
+                    double val = FULL ? full[(size_t)I * nc + j] : (slot >= 0 ? from[I] : E[a][ci]);
                     for (int l = 0; l < k; ++l) val -= jb.V[(size_t)l * nc + j] * jb.U[(size_t)l * m + I];
                     uk[I] = val;
                 }
@@ -209,6 +252,11 @@ __device__ void aca_block(const EntryGeo &g, const AcaJob &jb, AcaOut *out, doub
         }
         __syncthreads();
         if (threadIdx.x == 0) ucol[j] = 1;
+        if (keep && g.nin > 1 && cslot[j / g.nin] < 0 && ncs < ACA_KEEP) {
+            __syncthreads();
+            if (threadIdx.x == 0) cslot[j / g.nin] = (short)ncs;
+            ++ncs;
+        }
         // norms: ||u||^2, ||v||^2 and sum_l (u_l . u)(v_l . v)
         double pu = 0.0, pv = 0.0;
         for (int I = threadIdx.x; I < m; I += blockDim.x) pu += uk[I] * uk[I];
@@ -261,18 +309,19 @@ __device__ void aca_block(const EntryGeo &g, const AcaJob &jb, AcaOut *out, doub
     }
 }
 
-template <bool HALF, int THREADS>
-__global__ void __launch_bounds__(THREADS) aca_kernel(EntryGeo g, const AcaJob *jobs, AcaOut *outs, double eps) {
-    aca_block<HALF, THREADS, false>(g, jobs[blockIdx.x], outs + blockIdx.x, eps, nullptr);
-}
-
-// Small blocks, evaluated whole: persistent CTAs, each with one slot of `slot` doubles of scratch
-// (all of them together stay in L2).
-template <bool HALF, int THREADS>
-__global__ void __launch_bounds__(THREADS) aca_full_kernel(EntryGeo g, const AcaJob *jobs, AcaOut *outs, int njobs,
-                                                           double eps, double *scratch, int64_t slot) {
-    for (int b = blockIdx.x; b < njobs; b += gridDim.x) {
-        aca_block<HALF, THREADS, true>(g, jobs[b], outs + b, eps, scratch + blockIdx.x * slot);
+// Persistent CTAs, each with one slot of `slot` doubles of scratch for what its block keeps (FULL: the
+// block itself; those slots stay in L2 together), claiming the jobs in order.
+template <bool HALF, int THREADS, bool FULL>
+__global__ void __launch_bounds__(THREADS) aca_kernel(EntryGeo g, const AcaJob *jobs, AcaOut *outs, int njobs, double eps,
+                                                      double *scratch, int64_t slot, int *counter) {
+    __shared__ int s_job;
+    double *mine = scratch + blockIdx.x * slot;
+    for (;;) {
+        if (threadIdx.x == 0) s_job = atomicAdd(counter, 1);
+        __syncthreads();
+        const int b = s_job;
+        if (b >= njobs) return;
+        aca_block<HALF, THREADS, FULL>(g, jobs[b], outs + b, eps, FULL ? mine : nullptr, FULL || slot == 0 ? nullptr : mine);
         __syncthreads();
     }
 }
@@ -299,32 +348,38 @@ int aca_class(int tau, int sig, bool stepwise) {
     return side > 128 ? 0 : (side > 64 ? 1 : 2);
 }
 
-// ACA of jobs given by class (count[c] jobs of class c, in class order), the classes side by side
+// ACA of jobs given by class (count[c] jobs of class c, in class order, slot[c] doubles of scratch
+// for the largest), the classes side by side
 template <bool HALF>
-hbi_status launch_aca(const EntryGeo &g, const AcaJob *d_jobs, AcaOut *d_outs, const int *count, int64_t slot, int sms,
-                      double eps) {
-    BuildStreams bs;
+hbi_status launch_aca(const EntryGeo &g, const AcaJob *d_jobs, AcaOut *d_outs, const int *count, const int64_t *slot,
+                      int sms, double eps) {
     DevScratch tmp;
+    BuildStreams bs;
     hbi_status st = HBI_OK;
+    int *d_next = nullptr;
+    if ((st = tmp.alloc(&d_next, ACA_CLASSES * sizeof(int)))) return st;
+    HBI_CUDA_TRY(cudaMemset(d_next, 0, ACA_CLASSES * sizeof(int)));
     int at = 0;
     for (int c = 0; c < ACA_CLASSES; at += count[c], ++c) {
         if (count[c] == 0) continue;
         cudaStream_t s = nullptr;
         if ((st = bs.get(c, &s))) return st;
-        const AcaJob *j = d_jobs + at;
-        AcaOut *o = d_outs + at;
-        if (c == 0) aca_kernel<HALF, 256><<<(unsigned)count[c], 256, 0, s>>>(g, j, o, eps);
-        else if (c == 1) aca_kernel<HALF, 128><<<(unsigned)count[c], 128, 0, s>>>(g, j, o, eps);
-        else if (c == 2) aca_kernel<HALF, 64><<<(unsigned)count[c], 64, 0, s>>>(g, j, o, eps);
-        else {
+        auto launch = [&](auto *kernel, int threads) -> hbi_status {
             int occ = 1;
-            HBI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, aca_full_kernel<HALF, 64>, 64, 0));
+            HBI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, 0));
             const int grid = std::min(count[c], sms * std::max(1, occ));
             double *scratch = nullptr;
-            if ((st = tmp.alloc(&scratch, (size_t)grid * slot * sizeof(double)))) return st;
-            aca_full_kernel<HALF, 64><<<(unsigned)grid, 64, 0, s>>>(g, j, o, count[c], eps, scratch, slot);
-        }
-        HBI_CUDA_TRY(cudaGetLastError());
+            hbi_status a = tmp.alloc(&scratch, std::max<size_t>(1, (size_t)grid * slot[c]) * sizeof(double));
+            if (a) return a;
+            kernel<<<(unsigned)grid, threads, 0, s>>>(g, d_jobs + at, d_outs + at, count[c], eps, scratch, slot[c], d_next + c);
+            HBI_CUDA_TRY(cudaGetLastError());
+            return HBI_OK;
+        };
+        st = c == 0   ? launch(aca_kernel<HALF, 256, false>, 256)
+             : c == 1 ? launch(aca_kernel<HALF, 128, false>, 128)
+             : c == 2 ? launch(aca_kernel<HALF, 64, false>, 64)
+                      : launch(aca_kernel<HALF, 64, true>, 64);
+        if (st) return st;
     }
     return bs.wait();
 }
@@ -388,12 +443,15 @@ hbi_status device_build_factors(hbi_handle *h, const Tree &T, std::vector<Block>
             std::vector<AcaJob> sorted;
             std::vector<int> sorted_ids;
             int count[ACA_CLASSES] = {};
-            int64_t slot = 0;
+            int64_t slot[ACA_CLASSES] = {};
             for (int q : order) {
                 sorted.push_back(jobs[q]);
                 sorted_ids.push_back(ids[q]);
-                ++count[cls(q)];
-                if (cls(q) == 3) slot = std::max<int64_t>(slot, (int64_t)jobs[q].m * jobs[q].nc);
+                const AcaJob &J = jobs[q];
+                const int c = cls(q);
+                ++count[c];
+                slot[c] = std::max<int64_t>(slot[c], c == 3 ? (int64_t)J.m * J.nc
+                                                            : aca_keep_words(J.m, J.nc, J.tau_size, J.sig_size, h->nout, h->nin));
             }
             jobs.swap(sorted);
             ids.swap(sorted_ids);
