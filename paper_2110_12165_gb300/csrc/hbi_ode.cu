@@ -45,7 +45,7 @@ __global__ void prep_kernel(OdeArgs A) {
 // Stage s (0-based, 0..4) as its own launch: stage_elem over every element.
 __global__ void stage_kernel(OdeArgs A, int s) {
     if (all_stopped(A)) return;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += gridDim.x * blockDim.x) stage_elem(A, s, i);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += gridDim.x * blockDim.x) stage_elem<false>(A, s, i, nullptr);
 }
 
 // Stage 6 as its own launch (final_elem), with the per-model maxima of the error and of |V|
@@ -63,7 +63,7 @@ __global__ void final_kernel(OdeArgs A) {
     __syncthreads();
     if (i < n) {
         unsigned long long eb, vb, mu;
-        const int m = final_elem(A, i, eb, vb, mu);
+        const int m = final_elem<false>(A, i, nullptr, eb, vb, mu);
         if (m >= 0) {
             if (m - m0 < FINAL_SEG) {
                 atomicMax(&s_err[m - m0], eb);

@@ -101,16 +101,23 @@ __host__ __device__ __forceinline__ void stress_rates(const OdeArgs &A, int i, d
 }
 
 // dy/dt at element i for stage state (phi, tau, sig) with slip rate V and q = tau / sig
-// (Eqs. 8, 10, 12, 13)
-__host__ __device__ __forceinline__ void rhs_elem_q(const OdeArgs &A, int i, double phi, double V, double dVdtau,
-                                           double q, double &dphi, double &dtau, double &dsig) {
+// (Eqs. 8, 10, 12, 13): dphi needs the state alone, dtau and dsig the product's rows too
+__host__ __device__ __forceinline__ double rhs_dphi(const OdeArgs &A, int i, double phi, double V) {
+    return A.b_dc[i] * (A.V0 * exp((A.f0 - phi) * A.inv_b[i]) - V);   // Eq. 8
+}
+__host__ __device__ __forceinline__ void rhs_stress(const OdeArgs &A, int i, double V, double dVdtau, double q, double dphi,
+                                           double &dtau, double &dsig) {
     double AV, BV;
     stress_rates(A, i, AV, BV);
-    dphi = A.b_dc[i] * (A.V0 * exp((A.f0 - phi) * A.inv_b[i]) - V);   // Eq. 8
     dsig = BV;                                                          // Eq. 10 (+ loading)
     const double dVdsig = -q * dVdtau;                                  // Eq. 13b
     const double dVdphi = -V * A.inv_a[i];                              // Eq. 13c
     dtau = (AV - A.eta * (dVdsig * dsig + dVdphi * dphi)) / (1.0 + A.eta * dVdtau);   // Eq. 12
+}
+__host__ __device__ __forceinline__ void rhs_elem_q(const OdeArgs &A, int i, double phi, double V, double dVdtau,
+                                           double q, double &dphi, double &dtau, double &dsig) {
+    dphi = rhs_dphi(A, i, phi, V);
+    rhs_stress(A, i, V, dVdtau, q, dphi, dtau, dsig);
 }
 __host__ __device__ __forceinline__ void rhs_elem(const OdeArgs &A, int i, double phi, double tau, double sig, double V,
                                          double dVdtau, double &dphi, double &dtau, double &dsig) {

@@ -28,7 +28,45 @@ static __constant__ double c_B4[6] = {2825.0 / 27648.0, 0.0, 18575.0 / 48384.0, 
 // dV/dtau and tau/sigma kept beside it, and the next product input (V - V_pl) r into A.xt.
 // After a rejected attempt y is unchanged, so stage 0 keeps k_0 = f(y) from its slot (its
 // product was skipped) and only forms the stage inputs for the new step size.
-__device__ __forceinline__ void stage_elem(const OdeArgs &A, int s, int i) {
+//
+// With PRE, stage_pre has formed what does not need the product (dphi/dt and the sums over the
+// earlier stages; for stage 6 both solutions' sums), in the same order and to the same bits.  Inside
+// the UY launches it runs beside the streaming of the piece's rows, so that less is left when
+// they are written: an SM's FP64 pipe takes 16 cycles an instruction, and at the end of a launch
+// the last pieces of all its CTAs queue for it.
+struct StagePre {
+    double dphi, a[6];   // k_s's phi part; sums over l < s (stage 6: of order 5, then of order 4)
+};
+__device__ __forceinline__ void stage_pre(const OdeArgs &A, int s, int i, StagePre &P) {
+    const int n = A.n;
+    const StepCtl &C = A.ctl[A.model[i]];
+    if (C.stop) return;
+    if (!(s == 0 && C.reuse_k0)) P.dphi = rhs_dphi(A, i, A.ys[i], A.Vs[i]);
+    if (s < 5) {
+        double acc[3] = {0.0, 0.0, 0.0};
+        for (int l = 0; l < s; ++l) {
+            const double c = c_A[s + 1][l];
+            const double *kl = A.k + (size_t)l * 3 * n;
+            acc[0] += c * kl[i]; acc[1] += c * kl[n + i]; acc[2] += c * kl[2 * n + i];
+        }
+        P.a[0] = acc[0]; P.a[1] = acc[1]; P.a[2] = acc[2];
+        return;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        double s5 = 0.0, s4 = 0.0;
+#pragma unroll
+        for (int l = 0; l < 5; ++l) {
+            const double kv = A.k[(size_t)l * 3 * n + (size_t)c * n + i];
+            s5 += c_B5[l] * kv;
+            s4 += c_B4[l] * kv;
+        }
+        P.a[c] = s5;
+        P.a[3 + c] = s4;
+    }
+}
+template <bool PRE>
+__device__ __forceinline__ void stage_elem(const OdeArgs &A, int s, int i, const StagePre *P) {
     const int n = A.n;
     const StepCtl &C = A.ctl[A.model[i]];
     if (C.stop) return;
@@ -41,17 +79,26 @@ __device__ __forceinline__ void stage_elem(const OdeArgs &A, int s, int i) {
         for (int c = 0; c < A.nout; ++c)
             A.st_S[(size_t)s * A.nout * n + (size_t)A.nout * i + c] = read_y(A, (int64_t)A.nout * i + c);
     }
+    double kp, kt, ks;
     if (!keep_k0) {
-        double kp, kt, ks;
-        rhs_elem_q(A, i, A.ys[i], A.Vs[i], A.dVs[i], A.Vs[n + i], kp, kt, ks);
+        kp = PRE ? P->dphi : rhs_dphi(A, i, A.ys[i], A.Vs[i]);
+        rhs_stress(A, i, A.Vs[i], A.dVs[i], A.Vs[n + i], kp, kt, ks);
         ks_[i] = kp; ks_[n + i] = kt; ks_[2 * n + i] = ks;
+    } else {
+        kp = ks_[i]; kt = ks_[n + i]; ks = ks_[2 * n + i];
     }
     double acc[3] = {0.0, 0.0, 0.0};
-    for (int l = 0; l <= s; ++l) {
-        const double c = c_A[s + 1][l];
-        const double *kl = A.k + (size_t)l * 3 * n;
-        acc[0] += c * kl[i]; acc[1] += c * kl[n + i]; acc[2] += c * kl[2 * n + i];
+    if (PRE) {
+        for (int c = 0; c < 3; ++c) acc[c] = P->a[c];
+    } else {
+        for (int l = 0; l < s; ++l) {
+            const double c = c_A[s + 1][l];
+            const double *kl = A.k + (size_t)l * 3 * n;
+            acc[0] += c * kl[i]; acc[1] += c * kl[n + i]; acc[2] += c * kl[2 * n + i];
+        }
     }
+    const double cs = c_A[s + 1][s];
+    acc[0] += cs * kp; acc[1] += cs * kt; acc[2] += cs * ks;
     const double p1 = A.y[i] + dt * acc[0], t1 = A.y[n + i] + dt * acc[1], s1 = A.y[2 * n + i] + dt * acc[2];
     A.ys[i] = p1; A.ys[n + i] = t1; A.ys[2 * n + i] = s1;
     if (A.store) {
@@ -73,8 +120,9 @@ __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned
 // element's contributions to the model's reductions: the error and |V5| as the ordered bit
 // patterns of non-negative doubles, tau5/sigma5 in fixed point.  Returns the model index, or
 // -1 for an element of a stopped model (nothing written).
-__device__ __forceinline__ int final_elem(const OdeArgs &A, int i, unsigned long long &eb, unsigned long long &vb,
-                                          unsigned long long &mu) {
+template <bool PRE>
+__device__ __forceinline__ int final_elem(const OdeArgs &A, int i, const StagePre *P, unsigned long long &eb,
+                                          unsigned long long &vb, unsigned long long &mu) {
     const int n = A.n;
     const int m = A.model[i];
     StepCtl &C = A.ctl[m];
@@ -83,21 +131,27 @@ __device__ __forceinline__ int final_elem(const OdeArgs &A, int i, unsigned long
     if (A.store)
         for (int c = 0; c < A.nout; ++c)
             A.st_S[(size_t)5 * A.nout * n + (size_t)A.nout * i + c] = read_y(A, (int64_t)A.nout * i + c);
-    double kp, kt, ks;
-    rhs_elem_q(A, i, A.ys[i], A.Vs[i], A.dVs[i], A.Vs[n + i], kp, kt, ks);
+    const double kp = PRE ? P->dphi : rhs_dphi(A, i, A.ys[i], A.Vs[i]);
+    double kt, ks;
+    rhs_stress(A, i, A.Vs[i], A.dVs[i], A.Vs[n + i], kp, kt, ks);
     double *k5 = A.k + (size_t)5 * 3 * n;
     k5[i] = kp; k5[n + i] = kt; k5[2 * n + i] = ks;
+    const double kv5[3] = {kp, kt, ks};
     double y5[3], num = 0.0, den = 1.0;
     bool bad = false;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        double s5 = 0.0, s4 = 0.0;
+        double s5 = PRE ? P->a[c] : 0.0, s4 = PRE ? P->a[3 + c] : 0.0;
+        if (!PRE) {
 #pragma unroll
-        for (int l = 0; l < 6; ++l) {
-            const double kv = A.k[(size_t)l * 3 * n + (size_t)c * n + i];
-            s5 += c_B5[l] * kv;
-            s4 += c_B4[l] * kv;
+            for (int l = 0; l < 5; ++l) {
+                const double kv = A.k[(size_t)l * 3 * n + (size_t)c * n + i];
+                s5 += c_B5[l] * kv;
+                s4 += c_B4[l] * kv;
+            }
         }
+        s5 += c_B5[5] * kv5[c];
+        s4 += c_B4[5] * kv5[c];
         const double y0 = A.y[(size_t)c * n + i];
         y5[c] = y0 + dt * s5;
         const double y4 = y0 + dt * s4;
@@ -194,14 +248,17 @@ __device__ __forceinline__ int final_vec_elem(const OdeArgs &A, int i, unsigned 
 // first nthreads (a multiple of 32) threads of a CTA, each warp combining its lanes'
 // contributions when they all belong to one model (one atomic per quantity and warp), else
 // lane by lane.
+// pre (fixed rake, or nullptr): the elements' first parts.
 template <bool VEC>
-__device__ __forceinline__ void final_unit(const OdeArgs &A, int e0, int ne, int nthreads) {
+__device__ __forceinline__ void final_unit(const OdeArgs &A, int e0, int ne, int nthreads, const StagePre *pre) {
     const int lane = threadIdx.x & 31;
     for (int w0 = threadIdx.x - lane; w0 < ne; w0 += nthreads) {
         unsigned long long eb = 0ull, vb = 0ull, mu = 0ull;
         int m = -1;
         if (w0 + lane < ne)
-            m = VEC ? final_vec_elem(A, e0 + w0 + lane, eb, vb, mu) : final_elem(A, e0 + w0 + lane, eb, vb, mu);
+            m = VEC ? final_vec_elem(A, e0 + w0 + lane, eb, vb, mu)
+                    : (pre ? final_elem<true>(A, e0 + w0 + lane, pre + w0 + lane, eb, vb, mu)
+                           : final_elem<false>(A, e0 + w0 + lane, nullptr, eb, vb, mu));
         const int mlo = __reduce_min_sync(0xffffffffu, m < 0 ? INT_MAX : m), mhi = __reduce_max_sync(0xffffffffu, m);
         if (mhi < 0) continue;
         if (mlo == mhi) {
