@@ -204,6 +204,7 @@ struct VtBatch {
 // handle has one per model; each model keeps its own t, step size and decisions).
 struct StepCtl {
     double t, dt, dt_used, eps;
+    double dt_next; // the step control's next dt, formed beside the commit of the elements
     unsigned long long err_bits, vmax_bits;
     int accepted, target, rejects, stop, done_pending, status, accept_flag;
     int flags;      // bit 0: a trial had sigma <= 0, bit 1: a trial was non-finite
