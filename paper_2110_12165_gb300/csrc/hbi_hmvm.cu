@@ -393,8 +393,10 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
             fused_stage<FUSE>(ode, stage, prev_e0, prev_ne, 32 * FUSE_WARPS, ahead(prev_ne));
         prev_ne = 0;
         // and the first part of this piece's stage, thread e for element e
-        if (FUSE == 1 && warp < FUSE_WARPS && ahead(tk.rows / ode.nout) && (int)threadIdx.x < tk.rows / ode.nout)
-            stage_pre(ode, stage, (int)(tk.out_off / ode.nout) + threadIdx.x, s_pre[threadIdx.x]);
+        if (FUSE == 1 && warp < FUSE_WARPS) {
+            const PieceElems pe = piece_elems(tk, ode.nout, task_ok);
+            if (ahead(pe.ne) && (int)threadIdx.x < pe.ne) stage_pre(ode, stage, pe.e0 + threadIdx.x, s_pre[threadIdx.x]);
+        }
         if (rows_on) {
             // ---- rows: lanes split into groups of lpr per UY_RPW-row block, so that short rows
             //      still keep every lane busy (lpr, and with it each row's sum, is the same for
@@ -436,8 +438,9 @@ __global__ void __launch_bounds__(GEMV_THREADS, UyShape<UY_RPW>::blocks) uy_gemv
         }
         __syncthreads();
         if (FUSE) {   // the piece's elements (a skipped model's too: the stage decides)
-            prev_e0 = (int)(tk.out_off / ode.nout);
-            prev_ne = tk.rows / ode.nout;
+            const PieceElems pe = piece_elems(tk, ode.nout, task_ok);
+            prev_e0 = pe.e0;
+            prev_ne = pe.ne;
         }
     }
 }

@@ -175,6 +175,18 @@ struct GemvTask {
     int model;            // model of an ensemble handle the rows belong to
 };
 
+#ifdef __CUDACC__
+// The elements of a piece whose stage the UY launch may run: none of a record that the
+// bounds-checked build rejected (ok = false), whose rows were not computed and whose range may lie
+// outside the arrays the stage indexes.
+struct PieceElems {
+    int e0, ne;
+};
+__host__ __device__ __forceinline__ PieceElems piece_elems(const GemvTask &t, int nout, bool ok) {
+    return ok ? PieceElems{(int)(t.out_off / nout), t.rows / nout} : PieceElems{0, 0};
+}
+#endif
+
 // One VT-phase item: a row block x column chunk of the stacked V^T panel of a column group.
 // The panel (rows x cpad, row-major) and the x slice xt[x_off, x_off + cpad) are copied to
 // shared memory as they are; x_off is 16-byte aligned, so the group's columns sit at panel
