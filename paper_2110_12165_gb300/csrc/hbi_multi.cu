@@ -55,6 +55,7 @@ constexpr int MR_THREADS = 32 * (MR_GW + 2 + MR_BW);   // epilogue, A producer, 
 constexpr int MR_ROWS = 128;                       // MMA M: panel rows of a task
 constexpr int MR_A_STAGE = MR_ROWS * MR_CW * 2;    // bytes: one part (hi or lo) of a 128-row chunk
 constexpr int MR_KP_MAX = 64;                      // right-hand sides per call (padded to 16, 32 or 64)
+constexpr int MR_ZERO = 2 * MR_KP_MAX;             // halves before row 0 of x16: row -1 is zeros, whatever the row length
 constexpr int MR_KSLICE = 2048;                    // V^T: widest K of one task (wider groups are cut)
 constexpr unsigned long long MR_WAIT_NS = 1000000000ull;   // 1 s
 
@@ -91,7 +92,7 @@ struct hbi::MultiRhs {
     MrSplit *d_split = nullptr;   // V^T row tiles cut along K (reduced after the V^T phase)
     int n_split = 0;
     int64_t n_prow = 0;           // partial rows after T in xt
-    int *d_bidx = nullptr;        // B row indices of every task's chunks (rows of x16; padding: its zero row)
+    int *d_bidx = nullptr;        // B row indices of every task's chunks (rows of x16; padding: -1, its row of zeros)
     float *d_cscale = nullptr;    // per X row: the scale of its dense columns (largest over the blocks)
     int *d_iperm = nullptr;       // original element -> permuted position
     float *d_rowscale = nullptr;  // V^T output row scales (sv su)
@@ -102,9 +103,8 @@ struct hbi::MultiRhs {
     // per-call buffers, sized for kp_cap right-hand sides
     int kp_cap = 0;
     float *d_xt = nullptr, *d_yp = nullptr;
-    __half *d_x16 = nullptr;      // rows of X, of X with the dense column scales and of T, each [hi | lo], and a row of zeros
-    int row_kp = 0;               // the row length the grid and the row of zeros are for
-    int zeroed = 0;               // the row of zeros is written
+    __half *d_x16 = nullptr;      // MR_ZERO zeros, then rows of X, of X with the dense column scales and of T, each [hi | lo]
+    int row_kp = 0;               // the row length the grid is for
     unsigned *d_vmax = nullptr;   // per right-hand side: [0, 64) max |x|, [64, 128) max |t|,
                                   // [128, 192) max |x| x its row's dense column scale
     int *h_err = nullptr;         // error flag of bounded device waits (pinned; the kernels write it)
@@ -1010,7 +1010,7 @@ hbi_status pack_multi(hbi_handle *h, std::vector<Block> &blocks, const std::vect
     HBI_CUDA_TRY(cudaGetLastError());
     HBI_CUDA_TRY(cudaDeviceSynchronize());
 
-    // B row indices: MR_CW per chunk of every task, padding columns at the row of zeros after T
+    // B row indices: MR_CW per chunk of every task, padding columns at the row of zeros before X
     // (the row tiles of one leaf row unit share theirs)
     std::vector<int> bidx;
     int64_t last_gather = -1, last_off = 0;
@@ -1031,7 +1031,7 @@ hbi_status pack_multi(hbi_handle *h, std::vector<Block> &blocks, const std::vect
                 int64_t j = -1;
                 if (phase == 0) j = col < t.kreal ? gather + col : -1;
                 else if (col < end) j = gidx[gather + col];
-                bidx.push_back(j >= 0 ? (int)j : (int)(2 * M->nx + tcount));
+                bidx.push_back(j >= 0 ? (int)j : -1);
             }
         }
     };
@@ -1061,7 +1061,7 @@ hbi_status pack_multi(hbi_handle *h, std::vector<Block> &blocks, const std::vect
 namespace {
 hbi_status mr_prepare(hbi_handle *h, int kp) {
     MultiRhs *M = h->mr;
-    const int64_t rows16 = 2 * M->nx + M->n_t + 1;
+    const int64_t rows16 = 2 * M->nx + M->n_t;
     if (M->kp_cap < kp) {
         if (M->d_xt) cudaFree(M->d_xt);
         if (M->d_yp) cudaFree(M->d_yp);
@@ -1070,15 +1070,17 @@ hbi_status mr_prepare(hbi_handle *h, int kp) {
         M->d_x16 = nullptr;
         M->kp_cap = M->row_kp = 0;
         // xt rows: X, X scaled per row for the near field, T, partial rows of cut V^T tiles; x16
-        // rows: the first three, split, and one of zeros
+        // rows: the first three, split, behind the zeros, which are written here, once: no call
+        // writes there, so a call that fails (refused under stream capture) leaves them as they are
         HBI_ALLOC_TRY(&M->d_xt, (size_t)(2 * M->nx + M->n_t + M->n_prow) * kp * sizeof(float));
         HBI_ALLOC_TRY(&M->d_yp, (size_t)h->nout * h->n * kp * sizeof(float));
-        HBI_ALLOC_TRY(&M->d_x16, (size_t)rows16 * 2 * kp * sizeof(__half));
+        HBI_ALLOC_TRY(&M->d_x16, (MR_ZERO + (size_t)rows16 * 2 * kp) * sizeof(__half));
+        HBI_CUDA_TRY(cudaMemset(M->d_x16, 0, MR_ZERO * sizeof(__half)));
+        HBI_CUDA_TRY(cudaStreamSynchronize(nullptr));   // before any stream's product
         M->kp_cap = kp;
     }
     if (!M->d_vmax) HBI_ALLOC_TRY(&M->d_vmax, 192 * sizeof(unsigned));
-    if (M->row_kp != kp) {   // the row length, and with it the place of the row of zeros, goes with kp
-        M->zeroed = 0;
+    if (M->row_kp != kp) {
         const void *fn = mr_fn_for(kp);
         const int smem = mr_smem_bytes(kp);
         HBI_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -1119,12 +1121,12 @@ hbi_status mr_launch_phase(hbi_handle *h, int phase, cudaStream_t s) {
     auto split = [&](int vt, int64_t row0, int64_t nrows) {
         const int64_t blocks = (nrows * (KP / 8) + 255) / 256;
         return launch_dependent(mr_split_kernel<KP>, (int)std::max<int64_t>(1, std::min<int64_t>(blocks, 8 * sms)), 256, 0,
-                                s, M->d_xt, M->d_vmax, vt, row0, nrows, M->d_x16);
+                                s, M->d_xt, M->d_vmax, vt, row0, nrows, M->d_x16 + MR_ZERO);
     };
     if (phase == 0 && M->n_vt) {
         HBI_CUDA_TRY(split(1, 0, M->nx));
         HBI_CUDA_TRY(launch_dependent(mr_kernel<KP>, std::min(M->grid, M->n_vt), MR_THREADS, smem, s, M->d_vt, M->n_vt, 1,
-                                      M->d_panels, M->d_x16, M->d_bidx, M->d_rowscale, M->d_xt, M->d_vmax, M->h_err));
+                                      M->d_panels, M->d_x16 + MR_ZERO, M->d_bidx, M->d_rowscale, M->d_xt, M->d_vmax, M->h_err));
         if (M->n_split) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)M->n_split, MR_ROWS / MR_RED_ROWS);
@@ -1136,7 +1138,7 @@ hbi_status mr_launch_phase(hbi_handle *h, int phase, cudaStream_t s) {
     if (phase == 1 && M->n_uy) {
         HBI_CUDA_TRY(split(0, M->nx, M->nx + M->n_t));
         HBI_CUDA_TRY(launch_dependent(mr_kernel<KP>, std::min(M->grid, M->n_uy), MR_THREADS, smem, s, M->d_uy, M->n_uy, 0,
-                                      M->d_panels, M->d_x16, M->d_bidx, M->d_rowscale, M->d_yp, M->d_vmax, M->h_err));
+                                      M->d_panels, M->d_x16 + MR_ZERO, M->d_bidx, M->d_rowscale, M->d_yp, M->d_vmax, M->h_err));
     }
     return HBI_OK;
 }
@@ -1148,10 +1150,6 @@ hbi_status mr_phase(hbi_handle *h, int kp, int phase, cudaStream_t s) {
 hbi_status mr_enqueue(hbi_handle *h, int k, int kp, const double *d_X, double *d_Y, cudaStream_t s) {
     MultiRhs *M = h->mr;
     HBI_CUDA_TRY(cudaMemsetAsync(M->d_vmax, 0, 192 * sizeof(unsigned), s));
-    if (!M->zeroed) {
-        HBI_CUDA_TRY(cudaMemsetAsync(M->d_x16 + (2 * M->nx + M->n_t) * 2 * kp, 0, (size_t)2 * kp * sizeof(__half), s));
-        M->zeroed = 1;
-    }
     const int64_t ntile = ((int64_t)h->n + MR_TILE - 1) / MR_TILE, most = 8 * std::max(1, h->num_sms);
     const int gin = (int)std::min<int64_t>(ntile * h->nin, most), gout = (int)std::min<int64_t>(ntile * h->nout, most);
     hbi_status st = mr_dispatch(kp, [&](auto kc) -> hbi_status {
