@@ -272,16 +272,15 @@ __global__ void __launch_bounds__(THREADS, PER_SM) recompress_kernel(const Recom
 }
 
 namespace {
-template <int RMAX, int THREADS, int PER_SM>
-hbi_status recompress_class(const RecompJob *d_jobs, int *d_rank, int njobs, double tol, cudaStream_t s) {
-    if (njobs == 0) return HBI_OK;
-    const int smem = (6 * RMAX * RMAX + RC_TILE * RMAX + RMAX) * (int)sizeof(double);
-    auto *k = recompress_kernel<RMAX, THREADS, PER_SM>;
-    HBI_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    k<<<(unsigned)njobs, THREADS, smem, s>>>(d_jobs, d_rank, tol);
-    HBI_CUDA_TRY(cudaGetLastError());
-    return HBI_OK;
-}
+using RecompKernel = void (*)(const RecompJob *, int *, double);
+struct RecompClass {
+    RecompKernel kernel;
+    int rmax, threads;
+};
+constexpr int RC_CLASSES = 6;
+const RecompClass rc_classes[RC_CLASSES] = {{recompress_kernel<48, 192, 1>, 48, 192}, {recompress_kernel<40, 160, 2>, 40, 160},
+                                            {recompress_kernel<32, 128, 3>, 32, 128}, {recompress_kernel<24, 96, 6>, 24, 96},
+                                            {recompress_kernel<16, 64, 12>, 16, 64},  {recompress_kernel<8, 32, 16>, 8, 32}};
 }  // namespace
 
 // Recompress every low-rank block of rank 2..RC_RMAX; updates ranks in place (the first
@@ -300,7 +299,7 @@ hbi_status recompress_lowrank(std::vector<Block> &blocks, double tol) {
         const int cx = cls(x), cy = cls(y);
         return cx < cy || (cx == cy && blocks[x].m + blocks[x].nc > blocks[y].m + blocks[y].nc);
     });
-    int count[6] = {0, 0, 0, 0, 0, 0};
+    int count[RC_CLASSES] = {};
     for (int b : ids) {
         const Block &B = blocks[b];
         jobs.push_back(RecompJob{const_cast<double *>(B.d_src), const_cast<double *>(B.d_src2), (int)B.m, (int)B.nc,
@@ -312,25 +311,25 @@ hbi_status recompress_lowrank(std::vector<Block> &blocks, double tol) {
     DevScratch tmp;
     hbi_status st;
     if ((st = tmp.upload(&d_jobs, jobs)) || (st = tmp.alloc(&d_rank, jobs.size() * sizeof(int)))) return st;
-    BuildStreams bs;   // the classes side by side, so that one's last blocks do not leave SMs idle
-    int at = 0;
-    for (int c = 0; c < 6 && !st; at += count[c], ++c) {
-        const RecompJob *j = d_jobs + at;
-        int *r = d_rank + at;
-        cudaStream_t s = nullptr;
+    // the classes side by side, so that one's last blocks do not leave SMs idle; every kernel is loaded (on
+    // its first use, which waits for what is running) before the first launch
+    BuildStreams bs;
+    cudaStream_t stream[RC_CLASSES] = {};
+    int smem[RC_CLASSES] = {};
+    for (int c = 0; c < RC_CLASSES; ++c) {
         if (count[c] == 0) continue;
-        if ((st = bs.get(c, &s))) break;
-        switch (c) {
-            case 0: st = recompress_class<48, 192, 1>(j, r, count[c], tol, s); break;
-            case 1: st = recompress_class<40, 160, 2>(j, r, count[c], tol, s); break;
-            case 2: st = recompress_class<32, 128, 3>(j, r, count[c], tol, s); break;
-            case 3: st = recompress_class<24, 96, 6>(j, r, count[c], tol, s); break;
-            case 4: st = recompress_class<16, 64, 12>(j, r, count[c], tol, s); break;
-            default: st = recompress_class<8, 32, 16>(j, r, count[c], tol, s); break;
-        }
+        const int r = rc_classes[c].rmax;
+        smem[c] = (6 * r * r + RC_TILE * r + r) * (int)sizeof(double);
+        HBI_CUDA_TRY(cudaFuncSetAttribute(rc_classes[c].kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem[c]));
+        if ((st = bs.get(c, &stream[c]))) return st;
     }
-    const hbi_status st2 = bs.wait();
-    if (st || st2) return st ? st : st2;
+    int at = 0;
+    for (int c = 0; c < RC_CLASSES; at += count[c], ++c) {
+        if (count[c] == 0) continue;
+        rc_classes[c].kernel<<<(unsigned)count[c], rc_classes[c].threads, smem[c], stream[c]>>>(d_jobs + at, d_rank + at, tol);
+        HBI_CUDA_TRY(cudaGetLastError());
+    }
+    if ((st = bs.wait())) return st;
     std::vector<int> nr(jobs.size());
     HBI_CUDA_TRY(cudaMemcpy(nr.data(), d_rank, nr.size() * sizeof(int), cudaMemcpyDeviceToHost));
     for (size_t q = 0; q < jobs.size(); ++q) {
