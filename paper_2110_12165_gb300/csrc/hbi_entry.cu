@@ -53,17 +53,6 @@ struct AcaJob {
 // pair singular (which ACA need not meet)
 struct AcaOut { int rank, status; };
 
-// The entries are what ACA costs (a pair of elements takes about 2,000 FP64 instructions, and an
-// SM issues one FP64 warp instruction in 16 cycles), so a block gets the CTA that its larger side
-// fills, several of the small ones share an SM, and the largest blocks start first.  A block whose
-// pairs are fewer than ACA_DENSE rows and columns of them is evaluated whole before its ACA: a row
-// or column needs one of the pair's n_out rows or n_in columns but evaluates the pair, and its
-// last warp is mostly idle, so 24 rows and columns of a 40 x 40 block cost twice its 1,600 pairs.
-// With one 256-thread CTA (182 registers, one per SM) for every block, in partition order: 282
-// ms for the 9,086 blocks of a 20,022-element fault; so 134 ms one class
-// after the other, less side by side.
-constexpr int ACA_DENSE = 20;
-
 // block-wide argmax of (value, index) with ties to the smaller index; -1 if all excluded
 __device__ void block_argmax(double v, int idx, double *sv, int *si, double &best, int &bidx) {
     const int nw = blockDim.x >> 5;
@@ -337,15 +326,6 @@ hbi_status dev_alloc(T **p, size_t count, std::vector<void *> &owned) {
     owned.push_back(q);
     *p = (T *)q;
     return HBI_OK;
-}
-
-// The launch class of a block: 0-2 by the CTA its larger side fills (256, 128, 64 threads), 3
-// evaluated whole
-constexpr int ACA_CLASSES = 4;
-int aca_class(int tau, int sig, bool stepwise) {
-    if (!stepwise && ((int64_t)tau * sig + 31) / 32 <= ACA_DENSE * ((tau + 31) / 32 + (sig + 31) / 32)) return 3;
-    const int side = std::max(tau, sig);
-    return side > 128 ? 0 : (side > 64 ? 1 : 2);
 }
 
 // ACA of jobs given by class (count[c] jobs of class c, in class order, slot[c] doubles of scratch

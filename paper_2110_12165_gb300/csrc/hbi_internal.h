@@ -158,6 +158,33 @@ struct Block {
 std::vector<Block> build_partition(const Tree &T, int nin, int nout, double eta,
                                    std::vector<int> *lattice_ij = nullptr);
 
+// ------------------------------------------------------------ ACA launch classes
+// The entries are what ACA costs (a pair of elements takes about 2,000 FP64 instructions, and an
+// SM issues one FP64 warp instruction in 16 cycles), so a block gets the CTA that its larger side
+// fills, several of the small ones share an SM, and the largest blocks start first.  A block whose
+// pairs are fewer than ACA_DENSE rows and columns of them is evaluated whole before its ACA: a row
+// or column needs one of the pair's n_out rows or n_in columns but evaluates the pair, and its
+// last warp is mostly idle, so 24 rows and columns of a 40 x 40 block cost twice its 1,600 pairs.
+// With one 256-thread CTA (182 registers, one per SM) for every block, in partition order: 282
+// ms for the 9,086 blocks of a 20,022-element fault; so 134 ms one class
+// after the other, less side by side.
+// ACA_DENSE_SIDE bounds the longer side: a side of 20 elements or fewer passes the count against a
+// cluster of any size (a small fault beside a large one meets it whole), which one 64-thread
+// CTA would then evaluate alone: build of 4,000 elements and a fault of 16 far off 98 ms, of
+// 20,000 and 16 584 ms; with the bound 48 and 257.  48 to 128 measured the same on these, on twelve faults
+// of uneven size (35 ms, 44 without) and on 20,022 elements of one fault (221 ms with and without).
+constexpr int ACA_DENSE = 20, ACA_DENSE_SIDE = 128;
+constexpr int ACA_CLASSES = 4;
+// The launch class of a block of tau x sig elements: 0-2 by the CTA its larger side fills (256, 128, 64
+// threads), 3 evaluated whole (not when `stepwise`)
+inline int aca_class(int tau, int sig, bool stepwise) {
+    const int side = std::max(tau, sig);
+    if (!stepwise && side <= ACA_DENSE_SIDE &&
+        ((int64_t)tau * sig + 31) / 32 <= ACA_DENSE * ((tau + 31) / 32 + (sig + 31) / 32))
+        return 3;
+    return side > 128 ? 0 : (side > 64 ? 1 : 2);
+}
+
 // ------------------------------------------------------------ HMVM layout
 // One UY-phase work item (a leaf row unit or a piece of one): `rows` outputs, each the dot product of a stored
 // row with an input vector gathered into shared memory.  A row has two segments: dense
