@@ -299,7 +299,8 @@ __device__ void aca_block(const EntryGeo &g, const AcaJob &jb, AcaOut *out, doub
 }
 
 // Persistent CTAs, each with one slot of `slot` doubles of scratch for what its block keeps (FULL: the
-// block itself; those slots stay in L2 together), claiming the jobs in order.
+// block itself; those slots stay in L2 together; else nothing where the slot is too small), claiming
+// the jobs in order.
 template <bool HALF, int THREADS, bool FULL>
 __global__ void __launch_bounds__(THREADS) aca_kernel(EntryGeo g, const AcaJob *jobs, AcaOut *outs, int njobs, double eps,
                                                       double *scratch, int64_t slot, int *counter) {
@@ -310,7 +311,9 @@ __global__ void __launch_bounds__(THREADS) aca_kernel(EntryGeo g, const AcaJob *
         __syncthreads();
         const int b = s_job;
         if (b >= njobs) return;
-        aca_block<HALF, THREADS, FULL>(g, jobs[b], outs + b, eps, FULL ? mine : nullptr, FULL || slot == 0 ? nullptr : mine);
+        const AcaJob &J = jobs[b];
+        const bool fits = !FULL && aca_keep_words(J.m, J.nc, J.tau_size, J.sig_size, g.nout, g.nin) <= slot;
+        aca_block<HALF, THREADS, FULL>(g, J, outs + b, eps, FULL ? mine : nullptr, fits ? mine : nullptr);
         __syncthreads();
     }
 }
@@ -328,12 +331,12 @@ hbi_status dev_alloc(T **p, size_t count, std::vector<void *> &owned) {
     return HBI_OK;
 }
 
-// ACA of jobs given by class (count[c] jobs of class c, in class order, slot[c] doubles of scratch
+// ACA of jobs given by class (count[c] jobs of class c, in class order, want[c] doubles of scratch
 // for the largest), the classes side by side.  Every class's kernel is loaded and its scratch taken before
 // the first launch: a kernel's first use loads it, which waits for what is running (the first
 // half-space build of a process, 4,042 elements: 8.4 s loaded launch by launch, 4.0 s the later ones).
 template <bool HALF>
-hbi_status launch_aca(const EntryGeo &g, const AcaJob *d_jobs, AcaOut *d_outs, const int *count, const int64_t *slot,
+hbi_status launch_aca(const EntryGeo &g, const AcaJob *d_jobs, AcaOut *d_outs, const int *count, const int64_t *want,
                       int sms, double eps) {
     using Kernel = void (*)(EntryGeo, const AcaJob *, AcaOut *, int, double, double *, int64_t, int *);
     const Kernel kernel[ACA_CLASSES] = {aca_kernel<HALF, 256, false>, aca_kernel<HALF, 128, false>,
@@ -345,25 +348,28 @@ hbi_status launch_aca(const EntryGeo &g, const AcaJob *d_jobs, AcaOut *d_outs, c
     int *d_next = nullptr;
     if ((st = tmp.alloc(&d_next, ACA_CLASSES * sizeof(int)))) return st;
     HBI_CUDA_TRY(cudaMemset(d_next, 0, ACA_CLASSES * sizeof(int)));
-    int grid[ACA_CLASSES] = {};
+    AcaScratch plan[ACA_CLASSES] = {};
     double *scratch[ACA_CLASSES] = {};
     cudaStream_t stream[ACA_CLASSES] = {};
-    for (int c = 0; c < ACA_CLASSES; ++c) {
+    size_t free_b = 0, total_b = 0;
+    HBI_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+    int64_t left = (int64_t)(free_b / sizeof(double)) / ACA_SCRATCH_SHARE;
+    for (int c = ACA_CLASSES - 1; c >= 0; --c) {   // the many small blocks first
         if (count[c] == 0) continue;
         cudaFuncAttributes fa;
         HBI_CUDA_TRY(cudaFuncGetAttributes(&fa, kernel[c]));
         int occ = 1;
         HBI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel[c], threads[c], 0));
-        grid[c] = std::min(count[c], sms * std::max(1, occ));
-        if ((st = tmp.alloc(&scratch[c], std::max<size_t>(1, (size_t)grid[c] * slot[c]) * sizeof(double))) ||
+        plan[c] = aca_scratch(c, count[c], sms * std::max(1, occ), want[c], left);
+        if ((st = tmp.alloc(&scratch[c], std::max<size_t>(1, (size_t)plan[c].grid * plan[c].slot) * sizeof(double))) ||
             (st = bs.get(c, &stream[c])))
             return st;
     }
     int at = 0;
     for (int c = 0; c < ACA_CLASSES; at += count[c], ++c) {
         if (count[c] == 0) continue;
-        kernel[c]<<<(unsigned)grid[c], threads[c], 0, stream[c]>>>(g, d_jobs + at, d_outs + at, count[c], eps, scratch[c],
-                                                                   slot[c], d_next + c);
+        kernel[c]<<<(unsigned)plan[c].grid, threads[c], 0, stream[c]>>>(g, d_jobs + at, d_outs + at, count[c], eps,
+                                                                        scratch[c], plan[c].slot, d_next + c);
         HBI_CUDA_TRY(cudaGetLastError());
     }
     return bs.wait();
@@ -428,14 +434,14 @@ hbi_status device_build_factors(hbi_handle *h, const Tree &T, std::vector<Block>
             std::vector<AcaJob> sorted;
             std::vector<int> sorted_ids;
             int count[ACA_CLASSES] = {};
-            int64_t slot[ACA_CLASSES] = {};
+            int64_t want[ACA_CLASSES] = {};
             for (int q : order) {
                 sorted.push_back(jobs[q]);
                 sorted_ids.push_back(ids[q]);
                 const AcaJob &J = jobs[q];
                 const int c = cls(q);
                 ++count[c];
-                slot[c] = std::max<int64_t>(slot[c], c == 3 ? (int64_t)J.m * J.nc
+                want[c] = std::max<int64_t>(want[c], c == 3 ? (int64_t)J.m * J.nc
                                                             : aca_keep_words(J.m, J.nc, J.tau_size, J.sig_size, h->nout, h->nin));
             }
             jobs.swap(sorted);
@@ -461,8 +467,8 @@ hbi_status device_build_factors(hbi_handle *h, const Tree &T, std::vector<Block>
                 (st = tmp.alloc(&d_outs, jobs.size() * sizeof(AcaOut))))
                 return st;
             HBI_CUDA_TRY(cudaMemcpy(d_jobs, jobs.data(), jobs.size() * sizeof(AcaJob), cudaMemcpyHostToDevice));
-            if ((st = h->half_space ? launch_aca<true>(g, d_jobs, d_outs, count, slot, sms, eps)
-                                    : launch_aca<false>(g, d_jobs, d_outs, count, slot, sms, eps)))
+            if ((st = h->half_space ? launch_aca<true>(g, d_jobs, d_outs, count, want, sms, eps)
+                                    : launch_aca<false>(g, d_jobs, d_outs, count, want, sms, eps)))
                 return st;
             std::vector<AcaOut> outs(jobs.size());
             HBI_CUDA_TRY(cudaMemcpy(outs.data(), d_outs, outs.size() * sizeof(AcaOut), cudaMemcpyDeviceToHost));

@@ -185,6 +185,26 @@ inline int aca_class(int tau, int sig, bool stepwise) {
     return side > 128 ? 0 : (side > 64 ? 1 : 2);
 }
 
+// What a class's persistent CTAs get of the `left` doubles of scratch: `grid` CTAs with a slot of `slot`
+// doubles each (the class's largest block wants `want`).  A block of classes 0-2 whose components do
+// not fit its slot keeps none, at the cost of evaluating elements again; a block of class 3
+// needs its slot, so there are fewer CTAs.  ACA_SCRATCH_SHARE: of the memory that is free beside the batch's
+// factors, so that an operator is built wherever it is without the scratch (a class takes the slot
+// of its largest block for every CTA: 2.7 GB for blocks of 10,000 elements a side, 16 GB for
+// 60,000; the share of an empty 280 GB card is 17 GB).
+constexpr int64_t ACA_SCRATCH_SHARE = 16;
+struct AcaScratch {
+    int grid;
+    int64_t slot;
+};
+inline AcaScratch aca_scratch(int cls, int njobs, int resident, int64_t want, int64_t &left) {
+    AcaScratch s{std::max(1, std::min(njobs, resident)), want};
+    if (cls == 3) s.grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, left / std::max<int64_t>(1, want)));
+    else s.slot = std::min(want, left / s.grid);
+    left = std::max<int64_t>(0, left - s.grid * s.slot);
+    return s;
+}
+
 // ------------------------------------------------------------ HMVM layout
 // One UY-phase work item (a leaf row unit or a piece of one): `rows` outputs, each the dot product of a stored
 // row with an input vector gathered into shared memory.  A row has two segments: dense
