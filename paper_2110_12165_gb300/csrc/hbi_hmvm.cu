@@ -494,6 +494,11 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 constexpr unsigned long long VT_WAIT_NS = 1000000000ull;   // 1 s
+// A wait gave up: the host reads *err (its own memory, or the device's) once the stream is done.
+__device__ __forceinline__ void raise_error(int *err) {
+    *(volatile int *)err = 1;
+    __threadfence_system();
+}
 // One thread waits for the phase of the given parity; false once *fail is set or after VT_WAIT_NS.
 __device__ __forceinline__ bool thread_wait(uint64_t *bar, unsigned parity, volatile int *fail) {
     if (mbar_try_wait(bar, parity)) return true;   // already complete: no timer read
@@ -714,7 +719,7 @@ __global__ void __launch_bounds__(VT_THREADS, VT_CTAS_PER_SM) vt_stream_kernel(
             volatile int never = 0;
             for (int s = 0; s < min(n, VT_STAGES); ++s) {
                 mbar_arrive(&full[s]);
-                if (!thread_wait(&full[s], 0u, &never)) *fail = 1;
+                if (!thread_wait(&full[s], 0u, &never)) raise_error(err);   // the CTA returns below
             }
         }
 #else
@@ -812,10 +817,7 @@ __global__ void __launch_bounds__(VT_THREADS, VT_CTAS_PER_SM) vt_stream_kernel(
         }
     }
     __syncthreads();
-    if (tid == 0 && s_fail) {   // err may be host memory
-        *(volatile int *)err = 1;
-        __threadfence_system();
-    }
+    if (tid == 0 && s_fail) raise_error(err);
 }
 
 // A wait that can never complete (an mbarrier phase that expects one arrival nobody makes),
