@@ -1470,8 +1470,8 @@ hbi_status pack_operator(hbi_handle *h, const Tree *, std::vector<Block> &blocks
     }
     h->uy_rpw = h->uy_rpw_base = max_rows <= 8 ? 1 : (max_rows <= 16 ? 2 : 4);
     // every access of the two product kernels stays inside its buffers (the bounds-checked
-    // build checks the same limits on the device); a piece lies inside its unit and shares its
-    // gather list
+    // build checks the same limits on the device); the units' gather lists once, not again for
+    // every piece
     {
         TableLimits L;
         L.n_data1 = d1; L.n_data2 = d2; L.n_data3 = d3;
@@ -1481,7 +1481,8 @@ hbi_status pack_operator(hbi_handle *h, const Tree *, std::vector<Block> &blocks
         L.vt_panel_bytes = (int)VT_PANEL_BYTES; L.vt_x_bytes = (int)VT_X_BYTES; L.vt_max_sub = VT_MAX_SUB;
         L.vt_split_rows = VT_MC_ROWS;
         std::string first;
-        if (check_vt_tables(batches, items, L, &first) + check_uy_tables(units, gidx, L, &first) > 0) {
+        if (check_vt_tables(batches, items, L, &first) + check_uy_tables(units, gidx, L, &first) +
+                check_uy_pieces(units, t2, nout, &first) > 0) {
             set_error("internal error: an HMVM work table exceeds its buffers (" + first + ")");
             return HBI_ERR_INVALID_ARG;
         }

@@ -147,4 +147,36 @@ std::vector<Task> cut_uy_units(const std::vector<Task> &units, int nout, int es_
     return cut;
 }
 
+// The pieces that the UY kernel is given against the units that check_uy_tables has passed: in output
+// order they tile the units' rows, in whole elements, each with its unit's gather list and columns
+// and the stream offsets of its first row, so that every access of a piece is one of its unit's.
+template <typename Task>
+int64_t check_uy_pieces(std::vector<Task> units, std::vector<Task> pieces, int nout, std::string *first) {
+    using tables_detail::note;
+    auto by_row = [](const Task &a, const Task &b) { return a.out_off < b.out_off; };
+    std::sort(units.begin(), units.end(), by_row);
+    std::sort(pieces.begin(), pieces.end(), by_row);
+    int64_t bad = 0;
+    size_t pi = 0;
+    for (const Task &t : units) {
+        int64_t row = 0;
+        for (; row < t.rows && pi < pieces.size(); ++pi) {
+            const Task &c = pieces[pi];
+            const std::string where = "UY piece at output " + std::to_string(c.out_off) + ": ";
+            if (c.out_off != t.out_off + row || c.rows < 1 || c.rows > t.rows - row || c.rows % nout) {
+                note(bad, first, where + "rows");
+                return bad;
+            }
+            if (c.data_off != t.data_off + row * t.cpad || c.data_off_d != t.data_off_d + row * t.cpad_d)
+                note(bad, first, where + "stream offsets");
+            if (c.cpad != t.cpad || c.cpad_d != t.cpad_d || c.gather_off != t.gather_off || c.model != t.model)
+                note(bad, first, where + "columns");
+            row += c.rows;
+        }
+        if (row < t.rows) note(bad, first, "UY unit at output " + std::to_string(t.out_off) + ": rows without a piece");
+    }
+    if (pi < pieces.size()) note(bad, first, "UY pieces of no unit");
+    return bad;
+}
+
 }  // namespace hbi
