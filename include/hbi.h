@@ -231,7 +231,8 @@ hbi_status hbi_matvec_async(hbi_handle *h, const double *d_x, double *d_y, hbi_s
  * every GPU that loads the library holds until the process exits.  One product needs
  * 3 int words (work counter, error flag, finish count) plus (n_in N + T + 16) and n_out N accumulation
  * words (8 bytes for HBI_FP64 storage, 4 otherwise; T = sum of the ranks), each part rounded
- * up to 256 bytes; larger operators are rejected with HBI_ERR_INVALID_ARG.
+ * up to 256 bytes; larger operators are rejected with HBI_ERR_INVALID_ARG.  (The n_out N words are
+ * reserved: the product goes straight to d_y.)
  * The first call on a device looks the array's device address up (cudaGetSymbolAddress)
  * with that device current; make that first call before any stream capture.  Every call
  * shares the array, which keeps the last call's contents (each call clears the work counters

@@ -198,7 +198,7 @@ __device__ __forceinline__ A reduce_scatter(A (&v)[R], int sl, int lpr, int &row
 // is; each row's FMAs stay in column order.  FULL: nr == R; else the missing rows' loads are
 // predicated off, so that the last row block of a unit streams like the others and its partial
 // sums stay in registers (UY phase at N = 160,000: 475 us against 513 us with a loop over the
-// rows present, 96 % of the copy bandwidth).
+// rows present, 94 % of the copy bandwidth; 471 us, 95 %, with the units cut).
 template <int R, int UN, bool FULL, typename T>
 __device__ __forceinline__ void segment_steps(const T *__restrict__ rowp, int cpad, int nr,
                                               const typename Vec<T>::A *z, int c, int step,
@@ -1719,7 +1719,7 @@ struct NoallocRun {
         A *xt = reinterpret_cast<A *>(base + off);
         const size_t nxt = (size_t)h->nin * h->n + (size_t)h->n_t;
         off += align256((nxt + 16) * sizeof(A));
-        A *yp = reinterpret_cast<A *>(base + off);
+        A *yp = reinterpret_cast<A *>(base + off);   // reserved, not written: the UY phase writes y
         const int grid = std::max(1, std::min((h->n + 255) / 256, 4 * std::max(1, h->num_sms)));
         HBI_CUDA_TRY(cudaMemsetAsync(xt + nxt, 0, 16 * sizeof(A), s));   // guard elements
         HBI_CUDA_TRY(cudaMemsetAsync(counters, 0, 3 * sizeof(int), s));   // work counter, error flag, UY finish count

@@ -1181,6 +1181,9 @@ hbi_status mr_args(hbi_handle *h, int k, int &kp) {
         return HBI_ERR_INVALID_ARG;
     }
     if (k < 1 || k > MR_KP_MAX) { set_error("need 1 <= k <= 64 right-hand sides"); return HBI_ERR_INVALID_ARG; }
+    // 33 to 48 as 64: a third more row bytes and buffers than rows of 48 would take, which do not fill a
+    // swizzle row (k = 40 at 40,000 elements 362 us a call, 64 right-hand sides 370, 32 290; the
+    // kernel that converted gathered rows of 48 took 509)
     kp = k <= 16 ? 16 : (k <= 32 ? 32 : 64);
     if (h->num_sms <= 0) {
         int dev = 0;
@@ -1215,7 +1218,7 @@ extern "C" hbi_status hbi_time_multi(hbi_handle *h, int k, int n_rep, double *ou
     for (auto &x : e) HBI_CUDA_TRY(cudaEventCreate(&x));
     double acc[3] = {0, 0, 0};
     for (int r = 0; r < n_rep && !st; ++r) {
-        // the input already in xt (from the last call); the scales are recomputed from it
+        // the input already in xt and its scales (from the last call)
         HBI_CUDA_TRY(cudaEventRecord(e[0], s));
         st = mr_phase(h, kp, 0, s);
         if (!st) { HBI_CUDA_TRY(cudaEventRecord(e[1], s)); st = mr_phase(h, kp, 1, s); }
