@@ -566,10 +566,13 @@ constexpr int MR_TILE = 32;   // rows of the shared-memory transpose tiles of th
 // memory: read with consecutive threads on consecutive elements of one right-hand side
 // (coalesced, a thread's KP / 8 reads in flight together), written as whole rows of KP words at the
 // elements' permuted positions (iperm).  A thread writes one right-hand side throughout and keeps
-// its maxima in registers (one shared and one global atomic per right-hand side and block).
+// its maxima in registers (one shared and one global atomic per right-hand side and block).  Every
+// call writes the row of zeros (`zeros`, MR_ZERO halves) itself: nothing remembers that one has, so a call
+// that fails (refused under stream capture) leaves nothing wrong behind.
 template <int KP>
 __global__ void __launch_bounds__(256) mr_in_kernel(const double *X, const int *__restrict__ iperm, int n, int nin, int k,
-                                                    const float *__restrict__ cscale, float *xt, unsigned *vmax) {
+                                                    const float *__restrict__ cscale, float *xt, unsigned *vmax,
+                                                    uint4 *zeros) {
     __shared__ float tile[MR_TILE][KP + 1];
     __shared__ unsigned s_m[2][KP];
     constexpr int NL = KP * MR_TILE / 256;   // values of a tile per thread
@@ -578,6 +581,7 @@ __global__ void __launch_bounds__(256) mr_in_kernel(const double *X, const int *
     const int64_t ntile = ((int64_t)n + MR_TILE - 1) / MR_TILE * nin;
     for (int q = tid; q < 2 * KP; q += 256) s_m[q / KP][q % KP] = 0u;
     pdl_wait();
+    if (blockIdx.x == 0 && tid < MR_ZERO / 8) zeros[tid] = make_uint4(0u, 0u, 0u, 0u);
     float m = 0.0f, mc = 0.0f;
     const int jl = tid % MR_TILE, rr = tid / MR_TILE;   // reading: element, first right-hand side
     const int wr = tid % KP, wj = tid / KP;             // writing: right-hand side, first element
@@ -1070,13 +1074,10 @@ hbi_status mr_prepare(hbi_handle *h, int kp) {
         M->d_x16 = nullptr;
         M->kp_cap = M->row_kp = 0;
         // xt rows: X, X scaled per row for the near field, T, partial rows of cut V^T tiles; x16
-        // rows: the first three, split, behind the zeros, which are written here, once: no call
-        // writes there, so a call that fails (refused under stream capture) leaves them as they are
+        // rows: the first three, split, behind the row of zeros
         HBI_ALLOC_TRY(&M->d_xt, (size_t)(2 * M->nx + M->n_t + M->n_prow) * kp * sizeof(float));
         HBI_ALLOC_TRY(&M->d_yp, (size_t)h->nout * h->n * kp * sizeof(float));
         HBI_ALLOC_TRY(&M->d_x16, (MR_ZERO + (size_t)rows16 * 2 * kp) * sizeof(__half));
-        HBI_CUDA_TRY(cudaMemset(M->d_x16, 0, MR_ZERO * sizeof(__half)));
-        HBI_CUDA_TRY(cudaStreamSynchronize(nullptr));   // before any stream's product
         M->kp_cap = kp;
     }
     if (!M->d_vmax) HBI_ALLOC_TRY(&M->d_vmax, 192 * sizeof(unsigned));
@@ -1154,7 +1155,7 @@ hbi_status mr_enqueue(hbi_handle *h, int k, int kp, const double *d_X, double *d
     const int gin = (int)std::min<int64_t>(ntile * h->nin, most), gout = (int)std::min<int64_t>(ntile * h->nout, most);
     hbi_status st = mr_dispatch(kp, [&](auto kc) -> hbi_status {
         HBI_CUDA_TRY(launch_dependent(mr_in_kernel<decltype(kc)::value>, gin, 256, 0, s, d_X, M->d_iperm, h->n, h->nin, k,
-                                      M->d_cscale, M->d_xt, M->d_vmax));
+                                      M->d_cscale, M->d_xt, M->d_vmax, reinterpret_cast<uint4 *>(M->d_x16)));
         return HBI_OK;
     });
     if (st || (st = mr_phase(h, kp, 0, s)) || (st = mr_phase(h, kp, 1, s))) return st;
